@@ -80,6 +80,9 @@ struct rt_batch {
     std::vector<int64_t> chunk;                     // sources per chunk of each solve
     std::vector<int64_t> tlev;                      // per solve: levels that read tables in the last run
     BatchSolve* d_solves = nullptr;
+    std::vector<FieldJob> jobs;             // the solves' per-cell passes, then an end mark
+    FieldJob* d_jobs = nullptr;
+    uint32_t field_blocks = 0;
     DevStats* d_stats = nullptr;
     DevStats* h_stats = nullptr;           // pinned
     DevStats* m_stats = nullptr;           // its device address (mapped)
@@ -331,16 +334,7 @@ int enqueue(rt_batch* b)
 {
     cudaStream_t s = b->stream;
     b->launches = 0;
-    for (size_t i = 0; i < b->hs.size(); ++i) {
-        rt_handle* h = b->hs[i];
-        B_CUDA(b, cudaMemsetAsync(h->d_gamma, 0, sizeof(double) * (size_t)h->ncell, s), "gamma clear");
-        if (b->precision == RT_FP32)
-            b->launches += launch_prepare_kappa_f32(h->d_nh, h->d_x, h->ncell, h->sdx, b->n_th[i],
-                                                    static_cast<float*>(h->d_kap), s);
-        else
-            b->launches += launch_prepare_kappa_f64(h->d_nh, h->d_x, h->ncell, h->sdx, b->n_th[i],
-                                                    static_cast<double*>(h->d_kap), s);
-    }
+    b->launches += launch_prepare_many(b->d_jobs, (int)b->hs.size(), b->field_blocks, b->precision == RT_FP32, s);
     B_CUDA(b, cudaGetLastError(), "kappa launch");
     B_CUDA(b, cudaMemsetAsync(b->d_stats, 0, sizeof(DevStats) * b->hs.size(), s), "stats clear");
     B_CUDA(b, cudaMemsetAsync(b->d_err, 0, sizeof(unsigned), s), "error clear");
@@ -398,11 +392,7 @@ int enqueue(rt_batch* b)
         const int rc = enqueue_heavy(b, hv);
         if (rc) return rc;
     }
-    for (size_t i = 0; i < b->hs.size(); ++i) {
-        rt_handle* h = b->hs[i];
-        b->launches += launch_finalize(h->d_gamma, h->d_nh, h->d_x, h->ncell, h->cfg.e_heat_erg, h->vol, h->d_heat,
-                                       b->d_stats + i, s);
-    }
+    b->launches += launch_finalize_many(b->d_jobs, (int)b->hs.size(), b->field_blocks, s);
     B_CUDA(b, cudaGetLastError(), "finalize launch");
     // statistics and error word written into pinned memory by a kernel, not copied: a server's
     // result copies of the previous batch may occupy the copy engines
@@ -671,6 +661,8 @@ int nyx::batch_bind(rt_batch* b, rt_handle* const* handles, int32_t count)
         B_CUDA(b, cudaStreamSynchronize(b->stream), "batch stream");   // the pinned block is read on the host
         if (b->d_stats) B_CUDA(b, cudaFreeAsync(b->d_stats, b->stream), "stats");
         if (b->d_solves) B_CUDA(b, cudaFreeAsync(b->d_solves, b->stream), "solve table");
+        if (b->d_jobs) B_CUDA(b, cudaFreeAsync(b->d_jobs, b->stream), "field jobs");
+        b->d_jobs = nullptr;
         cudaFreeHost(b->h_stats);
         b->d_stats = nullptr;
         b->h_stats = nullptr;
@@ -681,8 +673,25 @@ int nyx::batch_bind(rt_batch* b, rt_handle* const* handles, int32_t count)
         B_CUDA(b, cudaMallocHost(&b->h_stats, sizeof(DevStats) * (size_t)b->cap_solves), "stats");
         B_CUDA(b, cudaHostGetDevicePointer(reinterpret_cast<void**>(&b->m_stats), b->h_stats, 0), "stats");
         B_CUDA(b, cudaMallocAsync(&b->d_solves, sizeof(BatchSolve) * (size_t)b->cap_solves, b->stream), "solve table");
+        B_CUDA(b, cudaMallocAsync(&b->d_jobs, sizeof(FieldJob) * (size_t)(b->cap_solves + 1), b->stream), "field jobs");
     }
     b->hsolve.assign(b->hs.size(), BatchSolve{});
+    b->jobs.clear();
+    b->field_blocks = 0;
+    for (size_t i = 0; i < b->hs.size(); ++i) {
+        FieldJob j = field_job(b->hs[i], b->hs[i]->d_x);
+        j.n_th = b->n_th[i];
+        j.chk = nullptr;
+        j.heat = b->hs[i]->d_heat;
+        j.st = b->d_stats + i;
+        j.block0 = b->field_blocks;
+        b->field_blocks += field_blocks(j.ncell);
+        b->jobs.push_back(j);
+    }
+    b->jobs.emplace_back();
+    b->jobs.back().block0 = b->field_blocks;
+    B_CUDA(b, cudaMemcpyAsync(b->d_jobs, b->jobs.data(), sizeof(FieldJob) * b->jobs.size(), cudaMemcpyHostToDevice,
+                              b->stream), "field jobs");
     int64_t first = 0;
     for (size_t i = 0; i < b->hs.size(); ++i) {
         rt_handle* h = b->hs[i];
@@ -735,6 +744,7 @@ int rt_batch_destroy(rt_batch* b)
     cudaFree(b->d_lane_count);
     if (b->stream) {
         if (b->d_solves) cudaFreeAsync(b->d_solves, b->stream);
+        if (b->d_jobs) cudaFreeAsync(b->d_jobs, b->stream);
         if (b->d_stats) cudaFreeAsync(b->d_stats, b->stream);
         if (b->d_src) cudaFreeAsync(b->d_src, b->stream);
         cudaStreamSynchronize(b->stream);

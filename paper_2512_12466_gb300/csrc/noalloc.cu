@@ -256,7 +256,8 @@ extern "C" int rt_step_noalloc(const rt_config* cfg, void* cuda_stream, const do
     c.overlap_mode = cfg->overlap_mode;
     c.hash = (cfg->flags & RT_FLAG_VISIT_HASH) ? 1 : 0;
     c.launches = 0;
-    double* scalar = reinterpret_cast<double*>(base + kOffScalar);
+    FieldCheck* chk = reinterpret_cast<FieldCheck*>(base + kOffScalar);
+    static_assert(sizeof(FieldCheck) <= 256, "the scalar slot");
 
     // the source workspace, carved from the array
     SourceWork w;
@@ -287,38 +288,40 @@ extern "C" int rt_step_noalloc(const rt_config* cfg, void* cuda_stream, const do
         return RT_OK;
     };
     if ((rc = cu(cudaMemsetAsync(c.st, 0, sizeof(DevStats), s), "rt_step_noalloc: statistics clear failed"))) return rc;
-    c.launches += launch_validate_fields(n_H, x_ion, ncell, c.st, s);
+    if ((rc = cu(cudaMemsetAsync(chk, 0, sizeof(FieldCheck), s), "rt_step_noalloc: clear failed"))) return rc;
+    c.launches += launch_check_fields(n_H, x_ion, ncell, nullptr, nullptr, false, chk, s);
     c.launches += launch_validate_sources(cell_ijk, ndot, nsrc, n, c.st, s);
     c.launches += launch_dedup_sort(w, nsrc, n, s);
-    const bool want_mean = cfg->n_th_cm3 < 0;
-    if (want_mean) {
-        if ((rc = cu(cudaMemsetAsync(scalar, 0, sizeof(double), s), "rt_step_noalloc: clear failed"))) return rc;
-        c.launches += launch_mean_nh(n_H, ncell, scalar, s);
-    }
     if ((rc = cu(cudaGetLastError(), "rt_step_noalloc: launch failed"))) return rc;
-    unsigned bad = 0;
+    unsigned bad = 0, bad_fields = 0;
     int32_t m32 = 0;
-    double sum_nh = 0.0;
     if ((rc = cu(cudaMemcpyAsync(&bad, &c.st->bad_input, sizeof(bad), cudaMemcpyDeviceToHost, s), "rt_step_noalloc: read failed"))) return rc;
     if (nsrc > 0 && (rc = cu(cudaMemcpyAsync(&m32, w.count, sizeof(m32), cudaMemcpyDeviceToHost, s), "rt_step_noalloc: read failed"))) return rc;
-    if (want_mean && (rc = cu(cudaMemcpyAsync(&sum_nh, scalar, sizeof(double), cudaMemcpyDeviceToHost, s), "rt_step_noalloc: read failed")))
+    if ((rc = cu(cudaMemcpyAsync(&bad_fields, &chk->bad, sizeof(bad_fields), cudaMemcpyDeviceToHost, s), "rt_step_noalloc: read failed")))
         return rc;
     if ((rc = cu(cudaStreamSynchronize(s), "rt_step_noalloc: source stage failed"))) return rc;
-    if (bad) return set_error(RT_EINVAL, "rt_step_noalloc: invalid field or source values");
+    if (bad || bad_fields) return set_error(RT_EINVAL, "rt_step_noalloc: invalid field or source values");
     const int64_t m = nsrc > 0 ? m32 : 0;
     c.n_emit = m;
     c.launches += launch_build_emit(w, m, cfg->sigma_cm2 / (dx * dx), emit, c.st, s);
-    const double n_th = want_mean ? 0.01 * (sum_nh / (double)ncell) : cfg->n_th_cm3;
-    const double sdx = cfg->sigma_cm2 * dx;
-    if (cfg->precision == RT_FP32)
-        c.launches += launch_prepare_kappa_f32(n_H, x_ion, ncell, sdx, n_th, reinterpret_cast<float*>(base + kOffKap), s);
-    else
-        c.launches += launch_prepare_kappa_f64(n_H, x_ion, ncell, sdx, n_th, reinterpret_cast<double*>(base + kOffKap), s);
-    if ((rc = cu(cudaMemsetAsync(gamma_out, 0, sizeof(double) * (size_t)ncell, s), "rt_step_noalloc: gamma clear failed"))) return rc;
+    FieldJob job;
+    job.nh = n_H;
+    job.x = x_ion;
+    job.kap = base + kOffKap;
+    job.gamma = gamma_out;
+    job.heat = heat_out;
+    job.ncell = ncell;
+    job.sdx = cfg->sigma_cm2 * dx;
+    job.n_th = cfg->n_th_cm3;
+    job.chk = cfg->n_th_cm3 < 0 ? chk : nullptr;
+    job.e_heat = cfg->e_heat_erg;
+    job.vol = dx * dx * dx;
+    job.st = c.st;
+    c.launches += launch_prepare_kappa(job, cfg->precision == RT_FP32, s);
     if ((rc = cu(cudaGetLastError(), "rt_step_noalloc: launch failed"))) return rc;
     rc = cfg->precision == RT_FP32 ? na_level<float>(c, 0, 0) : na_level<double>(c, 0, 0);
     if (rc) return rc;
-    c.launches += launch_finalize(gamma_out, n_H, x_ion, ncell, cfg->e_heat_erg, dx * dx * dx, heat_out, c.st, s);
+    c.launches += launch_finalize(job, s);
     if ((rc = cu(cudaGetLastError(), "rt_step_noalloc: finalize launch failed"))) return rc;
     DevStats d;
     if ((rc = cu(cudaMemcpyAsync(&d, c.st, sizeof(d), cudaMemcpyDeviceToHost, s), "rt_step_noalloc: stats read failed"))) return rc;

@@ -41,6 +41,7 @@ thread_local std::string g_create_error;
 constexpr int64_t kMaxChildrenPerLaunch = int64_t(1) << 27;
 constexpr int kMarchBlock = 256;
 constexpr int kMarchBlocksPerSm = 12;
+constexpr char kBadInput[] = "invalid field or source values (n_H < 0, x outside [0,1], non-finite, bad source)";
 
 struct DirTable {
     int level = -1;
@@ -702,17 +703,53 @@ int run_level(rt_handle* h, int level, int64_t nparents)
     return RT_OK;
 }
 
+FieldJob field_job(const rt_handle* h, const double* x)
+{
+    FieldJob j;
+    j.nh = h->d_nh;
+    j.x = x;
+    j.kap = h->d_kap;
+    j.gamma = h->d_gamma;
+    j.ncell = h->ncell;
+    j.sdx = h->sdx;
+    j.n_th = h->cfg.n_th_cm3;
+    j.chk = h->cfg.n_th_cm3 < 0 ? h->d_chk : nullptr;
+    j.e_heat = h->cfg.e_heat_erg;
+    j.vol = h->vol;
+    j.st = h->d_st;
+    return j;
+}
+
+int enqueue_field_check(rt_handle* h)
+{
+    const bool want_x = h->cfg.merge_mode == RT_MERGE_AUTO;
+    if (h->fields_checked && (h->checked_x || !want_x)) return RT_OK;
+    RT_CUDA(h, cudaMemsetAsync(h->d_chk, 0, sizeof(FieldCheck), h->stream), "check clear");
+    h->launches += launch_check_fields(h->d_nh, h->d_x, h->ncell, nullptr, nullptr, want_x, h->d_chk, h->stream);
+    RT_LAUNCHED(h, "check launch");
+    h->fields_checked = true;
+    h->checked_x = want_x;
+    return RT_OK;
+}
+
+// A caller's buffer that a kernel on the handle's device may read or write itself: aligned memory of
+// that device. Everything else (host, managed or another device's memory) goes through a copy.
+bool direct_access(const rt_handle* h, const void* p)
+{
+    cudaPointerAttributes a;
+    if (reinterpret_cast<uintptr_t>(p) & 7) return false;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return a.type == cudaMemoryTypeDevice && a.device == h->device;
+}
+
 int trace(rt_handle* h, const double* xuse)
 {
-    RT_CUDA(h, cudaMemsetAsync(h->d_gamma, 0, sizeof(double) * (size_t)h->ncell, h->stream), "gamma clear");
     // per-trace part of the statistics: per-level counters, hash and ledger
     RT_CUDA(h, cudaMemsetAsync(h->d_st, 0, offsetof(DevStats, deposited), h->stream), "stats clear");
-    double n_th = h->cfg.n_th_cm3;
-    if (n_th < 0) n_th = 0.01 * h->h_f64[1];
-    if (h->cfg.precision == RT_FP32)
-        launch_prepare_kappa_f32(h->d_nh, xuse, h->ncell, h->sdx, n_th, static_cast<float*>(h->d_kap), h->stream);
-    else
-        launch_prepare_kappa_f64(h->d_nh, xuse, h->ncell, h->sdx, n_th, static_cast<double*>(h->d_kap), h->stream);
+    launch_prepare_kappa(field_job(h, xuse), h->cfg.precision == RT_FP32, h->stream);
     RT_LAUNCHED(h, "kappa launch");
     h->launches++;
     h->march_launches = 0;
@@ -727,7 +764,7 @@ int trace(rt_handle* h, const double* xuse)
 
 // Sec. 2.8 source stage of a step: validation of device-resident inputs,
 // dedup + sort, the n_th default, Alg. 3 merging when on, and the emitted
-// catalog (h->d_emit, h->n_emit). Leaves h->h_f64[1] = mean n_H (default n_th).
+// catalog (h->d_emit, h->n_emit). Leaves the field check in h->h_chk.
 int prepare_sources(rt_handle* h, bool* merged_out, int64_t* n_dedup_out)
 {
     NvtxRange nvtx("source stage (dedup, sort, Alg. 3)");
@@ -735,31 +772,25 @@ int prepare_sources(rt_handle* h, bool* merged_out, int64_t* n_dedup_out)
     *merged_out = false;
     h->catalog_valid = false;            // the buffers below are rewritten; valid again once emitted
     // ---- validation of device-resident inputs
-    h->launches += launch_validate_fields(h->d_nh, h->d_x, h->ncell, h->d_st, s);
+    {
+        const int rc = enqueue_field_check(h);
+        if (rc) return rc;
+    }
     h->launches += launch_validate_sources(h->sw.cells_raw, h->sw.ndot_raw, h->nsrc, h->cfg.n, h->d_st, s);
     RT_LAUNCHED(h, "validation launch");
 
     // ---- sources: dedup + sort (Sec. 2.8)
     h->launches += launch_dedup_sort(h->sw, h->nsrc, h->cfg.n, s);
     RT_LAUNCHED(h, "source launch");
-    bool want_mean_nh = h->cfg.n_th_cm3 < 0;
-    if (want_mean_nh) {
-        RT_CUDA(h, cudaMemsetAsync(h->d_scalar, 0, sizeof(double), s), "scalar clear");
-        h->launches += launch_mean_nh(h->d_nh, h->ncell, h->d_scalar, s);
-    }
-    if (h->cfg.merge_mode == RT_MERGE_AUTO) h->launches += launch_sum_x(h->d_x, h->ncell, h->d_st, s);
-    RT_LAUNCHED(h, "reduction launch");
     RT_CUDA(h, cudaMemcpyAsync(h->h_st, h->d_st, sizeof(DevStats), cudaMemcpyDeviceToHost, s), "stats read");
     if (h->nsrc > 0)
         RT_CUDA(h, cudaMemcpyAsync(h->h_i32, h->sw.count, sizeof(int32_t), cudaMemcpyDeviceToHost, s), "count read");
-    if (want_mean_nh)
-        RT_CUDA(h, cudaMemcpyAsync(h->h_f64, h->d_scalar, sizeof(double), cudaMemcpyDeviceToHost, s), "mean read");
+    RT_CUDA(h, cudaMemcpyAsync(h->h_chk, h->d_chk, sizeof(FieldCheck), cudaMemcpyDeviceToHost, s), "check read");
     RT_CUDA(h, cudaStreamSynchronize(s), "source stage");
-    if (h->h_st->bad_input) return fail(h, RT_EINVAL, "invalid field or source values (n_H < 0, x outside [0,1], non-finite, bad source)");
-    h->h_f64[1] = want_mean_nh ? h->h_f64[0] / (double)h->ncell : 0.0;
+    if (h->h_st->bad_input || h->h_chk->bad) return fail(h, RT_EINVAL, kBadInput);
     int64_t m = h->nsrc > 0 ? h->h_i32[0] : 0;
     *n_dedup_out = m;
-    const double xbar = h->h_st->xsum / (double)h->ncell;
+    const double xbar = h->h_chk->sum_x / (double)h->ncell;
 
     // ---- Alg. 3 source merging
     if (m > 0 && (h->cfg.merge_mode == RT_MERGE_FORCED ||
@@ -817,20 +848,19 @@ int sources_enqueue_many(rt_handle* const* hs, int count, int* rcs)
         h->launches = 0;
         h->catalog_valid = false;
         RT_CUDA(h, cudaMemsetAsync(h->d_st, 0, sizeof(DevStats), s), "stats clear");
-        h->launches += launch_validate_fields(h->d_nh, h->d_x, h->ncell, h->d_st, s);
+        {
+            const int rc = enqueue_field_check(h);
+            if (rc) return rc;
+        }
         h->launches += launch_validate_sources(h->sw.cells_raw, h->sw.ndot_raw, h->nsrc, h->cfg.n, h->d_st, s);
         h->launches += launch_dedup_sort(h->sw, h->nsrc, h->cfg.n, s);
-        if (h->cfg.n_th_cm3 < 0) {
-            RT_CUDA(h, cudaMemsetAsync(h->d_scalar, 0, sizeof(double), s), "scalar clear");
-            h->launches += launch_mean_nh(h->d_nh, h->ncell, h->d_scalar, s);
-        }
         if (h->nsrc > 0) h->launches += launch_build_emit_dev(h->sw, h->nsrc, h->s_over_dx2, h->d_emit, h->d_st, s);
         // statistics, count and mean written into the pinned block by a kernel (a server's result
         // copies of other requests may occupy the copy engines)
         ReadbackList rb;
         rb.add(h->d_st, pinned_dev(h, h->h_st), sizeof(DevStats));
         if (h->nsrc > 0) rb.add(h->sw.count, pinned_dev(h, h->h_i32), sizeof(int32_t));
-        if (h->cfg.n_th_cm3 < 0) rb.add(h->d_scalar, pinned_dev(h, h->h_f64), sizeof(double));
+        rb.add(h->d_chk, pinned_dev(h, h->h_chk), sizeof(FieldCheck));
         h->launches += launch_readback(rb, s);
         RT_LAUNCHED(h, "source stage launch");
         return RT_OK;
@@ -853,8 +883,7 @@ int sources_wait_many(rt_handle* const* hs, int count, int* rcs)
         rt_handle* h = hs[i];
         if (rcs[i] == RT_OK && !h->src_ready) {
             if (cudaStreamSynchronize(h->stream) != cudaSuccess) rcs[i] = cuda_fail(h, cudaGetLastError(), "source stage");
-            else if (h->h_st->bad_input)
-                rcs[i] = fail(h, RT_EINVAL, "invalid field or source values (n_H < 0, x outside [0,1], non-finite, bad source)");
+            else if (h->h_st->bad_input || h->h_chk->bad) rcs[i] = fail(h, RT_EINVAL, kBadInput);
         }
         if (rcs[i] != RT_OK) { ++failed; continue; }
         if (h->src_ready) continue;
@@ -864,7 +893,7 @@ int sources_wait_many(rt_handle* const* hs, int count, int* rcs)
         h->src_ready = true;
         h->src_merged = false;
         h->src_dedup = m;
-        h->src_nth = h->cfg.n_th_cm3 >= 0 ? h->cfg.n_th_cm3 : 0.01 * (h->h_f64[0] / (double)h->ncell);
+        h->src_nth = h->cfg.n_th_cm3 >= 0 ? h->cfg.n_th_cm3 : h->h_chk->n_th;
         h->src_emitted = h->h_st->emitted;
     }
     return failed;
@@ -885,7 +914,7 @@ int handle_prepare_sources(rt_handle* h)
     h->src_ready = true;
     h->src_merged = merged;
     h->src_dedup = nd;
-    h->src_nth = h->cfg.n_th_cm3 >= 0 ? h->cfg.n_th_cm3 : 0.01 * h->h_f64[1];
+    h->src_nth = h->cfg.n_th_cm3 >= 0 ? h->cfg.n_th_cm3 : h->h_chk->n_th;
     h->src_emitted = h->h_st->emitted;
     return RT_OK;
 }
@@ -997,7 +1026,7 @@ int rt_destroy(rt_handle* h)
     DeviceGuard g(h->device);
     cudaStreamSynchronize(h->stream);
     {
-        void* ps[] = {h->d_nh, h->d_x, h->d_xavg, h->d_xend, h->d_gamma, h->d_heat, h->d_kap, h->d_scalar,
+        void* ps[] = {h->d_nh, h->d_x, h->d_xavg, h->d_xend, h->d_gamma, h->d_heat, h->d_kap, h->d_chk,
                       h->d_emit, h->d_count, h->d_st};
         for (void* q : ps) dfree(h, q);
         SourceWork& w = h->sw;
@@ -1039,13 +1068,13 @@ int rt_create(const rt_config* cfg, void* cuda_stream, rt_handle** out)
         e = e ? e : dalloc(h, (void**)&h->d_xavg, fb);
         e = e ? e : dalloc(h, (void**)&h->d_xend, fb);
     }
-    e = e ? e : dalloc(h, (void**)&h->d_scalar, 64);
+    e = e ? e : dalloc(h, (void**)&h->d_chk, sizeof(FieldCheck));
     e = e ? e : dalloc(h, (void**)&h->d_count, sizeof(unsigned long long) * (RT_MAX_LEVELS + 1));
     e = e ? e : dalloc(h, (void**)&h->d_st, sizeof(DevStats));
     {   // one pinned block for every host-side readback
         const size_t a = (sizeof(DevStats) + 63) & ~size_t(63);
         const size_t b = (sizeof(unsigned long long) * (RT_MAX_LEVELS + 1) + 63) & ~size_t(63);
-        e = e ? e : cudaMallocHost(&h->h_pin, a + b + 128);
+        e = e ? e : cudaMallocHost(&h->h_pin, a + b + 192);
         e = e ? e : cudaHostGetDevicePointer(reinterpret_cast<void**>(&h->d_pin), h->h_pin, 0);
         if (e == cudaSuccess) {
             char* q = static_cast<char*>(h->h_pin);
@@ -1053,6 +1082,7 @@ int rt_create(const rt_config* cfg, void* cuda_stream, rt_handle** out)
             h->h_count = reinterpret_cast<unsigned long long*>(q + a);
             h->h_i32 = reinterpret_cast<int32_t*>(q + a + b);
             h->h_f64 = reinterpret_cast<double*>(q + a + b + 64);
+            h->h_chk = reinterpret_cast<FieldCheck*>(q + a + b + 128);
         }
     }
     for (auto& ev : h->ev) e = e ? e : cudaEventCreate(&ev);
@@ -1073,6 +1103,18 @@ int rt_set_fields(rt_handle* h, const double* n_H, const double* x_ion, int wher
     if (h->sticky) return RT_ESTATE;
     DeviceGuard g(h->device);
     const size_t fb = sizeof(double) * (size_t)h->ncell;
+    h->fields_checked = false;
+    if (where == RT_DEVICE && direct_access(h, n_H) && direct_access(h, x_ion)) {
+        // copied and checked in one pass
+        const bool want_x = h->cfg.merge_mode == RT_MERGE_AUTO;
+        RT_CUDA(h, cudaMemsetAsync(h->d_chk, 0, sizeof(FieldCheck), h->stream), "check clear");
+        launch_check_fields(n_H, x_ion, h->ncell, h->d_nh, h->d_x, want_x, h->d_chk, h->stream);
+        RT_LAUNCHED(h, "field copy");
+        h->fields_checked = true;
+        h->checked_x = want_x;
+        h->fields_set = true;
+        return RT_OK;
+    }
     const cudaMemcpyKind k = where == RT_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
     RT_CUDA(h, cudaMemcpyAsync(h->d_nh, n_H, fb, k, h->stream), "field copy");
     RT_CUDA(h, cudaMemcpyAsync(h->d_x, x_ion, fb, k, h->stream), "field copy");
@@ -1311,18 +1353,16 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
     double resid = 0.0;
     const double* xuse = h->d_x;
     if (h->cfg.chem_iterate) {
-        RT_CUDA(h, cudaMemcpyAsync(h->d_xavg, h->d_x, sizeof(double) * (size_t)h->ncell, cudaMemcpyDeviceToDevice, s), "x copy");
-        xuse = h->d_xavg;
         const int maxit = h->cfg.chem_max_iter > 0 ? h->cfg.chem_max_iter : 100;
+        // the trace uses <x> in xuse (x itself at first) and the update writes the new <x> beside it: the
+        // one the last trace used stays, for the heating
+        double* xnew = h->d_xavg;
         for (;;) {
-            int rc = trace(h, h->d_xavg);
+            int rc = trace(h, xuse);
             if (rc) return rc;
             ++iters;
-            // the update overwrites <x>; keep the traced one for heating until convergence is known
-            RT_CUDA(h, cudaMemcpyAsync(h->d_heat, h->d_xavg, sizeof(double) * (size_t)h->ncell, cudaMemcpyDeviceToDevice, s),
-                    "x copy");
             RT_CUDA(h, cudaMemsetAsync(&h->d_st->maxdiff, 0, sizeof(double), s), "clear");
-            h->launches += launch_chem_update(h->d_nh, h->d_x, h->d_xavg, h->d_xend, h->d_gamma, h->ncell, dt_s,
+            h->launches += launch_chem_update(h->d_nh, h->d_x, xuse, xnew, h->d_xend, h->d_gamma, h->ncell, dt_s,
                                               h->cfg.alpha_B, h->cfg.C_H, h->cfg.clumping, h->d_st, s);
             RT_LAUNCHED(h, "chemistry launch");
             RT_CUDA(h, cudaMemcpyAsync(h->h_f64 + 2, &h->d_st->maxdiff, sizeof(double), cudaMemcpyDeviceToHost, s),
@@ -1330,27 +1370,37 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
             RT_CUDA(h, cudaStreamSynchronize(s), "chemistry");
             resid = h->h_f64[2];
             if (resid < h->cfg.chem_tol || iters >= maxit) break;
+            xuse = xnew;
+            xnew = xnew == h->d_xavg ? h->d_heat : h->d_xavg;
         }
-        // heating uses the <x> the last trace used (saved in d_heat); new x = x(t + dt)
-        std::swap(h->d_xavg, h->d_heat);
-        xuse = h->d_xavg;
+        // heating uses the <x> the last trace used; it may be d_heat, which then takes the other's place
+        if (xuse == h->d_heat) std::swap(h->d_xavg, h->d_heat);
     } else {
         int rc = trace(h, h->d_x);
         if (rc) return rc;
         iters = 1;
     }
 
-    // ---- heating, deposited photons
-    RT_CUDA(h, cudaMemsetAsync(&h->d_st->deposited, 0, sizeof(double), s), "clear");
-    h->launches += launch_finalize(h->d_gamma, h->d_nh, xuse, h->ncell, h->cfg.e_heat_erg, h->vol, h->d_heat, h->d_st, s);
-    RT_LAUNCHED(h, "finalize launch");
-    if (h->cfg.chem_iterate)
-        RT_CUDA(h, cudaMemcpyAsync(h->d_x, h->d_xend, sizeof(double) * (size_t)h->ncell, cudaMemcpyDeviceToDevice, s),
-                "x update");
+    // ---- heating, deposited photons, and the results straight into the caller's device buffers (a copy
+    // where a kernel may not write them, or where they overlap)
     const size_t fb = sizeof(double) * (size_t)h->ncell;
+    const char* const pg = reinterpret_cast<const char*>(gamma_out);
+    const char* const ph = reinterpret_cast<const char*>(heat_out);
+    const bool apart = !pg || !ph || pg + fb <= ph || ph + fb <= pg;
+    const bool gamma_direct = gamma_out && where == RT_DEVICE && apart && direct_access(h, gamma_out);
+    const bool heat_direct = heat_out && where == RT_DEVICE && apart && direct_access(h, heat_out);
+    FieldJob job = field_job(h, xuse);
+    job.gamma_out = gamma_direct ? gamma_out : nullptr;
+    job.heat = heat_direct ? heat_out : (heat_out ? h->d_heat : nullptr);
+    h->launches += launch_finalize(job, s);
+    RT_LAUNCHED(h, "finalize launch");
+    if (h->cfg.chem_iterate) {
+        std::swap(h->d_x, h->d_xend);         // x(t + dt)
+        h->fields_checked = false;
+    }
     const cudaMemcpyKind k = where == RT_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
-    if (gamma_out) RT_CUDA(h, cudaMemcpyAsync(gamma_out, h->d_gamma, fb, k, s), "gamma copy");
-    if (heat_out) RT_CUDA(h, cudaMemcpyAsync(heat_out, h->d_heat, fb, k, s), "heat copy");
+    if (gamma_out && !gamma_direct) RT_CUDA(h, cudaMemcpyAsync(gamma_out, h->d_gamma, fb, k, s), "gamma copy");
+    if (heat_out && !heat_direct) RT_CUDA(h, cudaMemcpyAsync(heat_out, h->d_heat, fb, k, s), "heat copy");
     RT_CUDA(h, cudaEventRecord(h->ev[3], s), "event");
     RT_CUDA(h, cudaMemcpyAsync(h->h_st, h->d_st, sizeof(DevStats), cudaMemcpyDeviceToHost, s), "stats read");
     RT_CUDA(h, cudaStreamSynchronize(s), "step");

@@ -105,7 +105,9 @@ struct rt_handle {
     double* d_gamma = nullptr;
     double* d_heat = nullptr;
     void* d_kap = nullptr;
-    double* d_scalar = nullptr;           // reduction scratch
+    nyx::FieldCheck* d_chk = nullptr;     // of d_nh and d_x, while fields_checked
+    bool fields_checked = false;          // the check has run (or is enqueued) on the fields as they are
+    bool checked_x = false;               // with the sum of x
 
     nyx::SourceWork sw;
     int64_t nsrc = 0;
@@ -122,6 +124,7 @@ struct rt_handle {
     unsigned long long* h_count = nullptr;
     int32_t* h_i32 = nullptr;                // scratch
     double* h_f64 = nullptr;                 // scratch
+    nyx::FieldCheck* h_chk = nullptr;
 
     cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     double ms_march = 0.0;
@@ -158,6 +161,10 @@ bool geometry_level(int device, long long rq, int level, int n, long long rs, co
                     cudaStream_t s, bool fp64, GeomLevel* out);
 // The RT_SPECTRUM_BLACKBODY tables at t_bb for `device` (device < 0: host table only).
 int spectrum_table(int device, double t_bb, SpecTable<double>* d, SpecTable<float>* f, std::string& why);
+// The field check of a handle, enqueued if its fields have not been checked yet.
+int enqueue_field_check(rt_handle* h);
+// The job of a handle's per-cell passes (x: the ionized fraction to use).
+FieldJob field_job(const rt_handle* h, const double* x);
 int handle_prepare_sources(rt_handle* h);
 int handle_reconfigure(rt_handle* h, const rt_config* cfg);
 int sources_enqueue_many(rt_handle* const* hs, int count, int* rcs);

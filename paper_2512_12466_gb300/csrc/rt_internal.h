@@ -44,9 +44,32 @@ struct DevStats {
     double deposited;
     double emitted;
     double maxdiff;                  // chemistry: max |<x>_new - <x>_old| (as ordered bits)
-    double xsum;                     // sum of x (automerge)
     unsigned int err;                // RT_ERR_* bits set by kernels
     unsigned int bad_input;          // count of invalid field / source values
+};
+
+// What one pass over a handle's fields finds.
+struct FieldCheck {
+    double sum_nh, sum_x;
+    double n_th;                     // default threshold of Eqs. 7-8: 0.01 mean(n_H)
+    unsigned bad;                    // cells with n_H < 0, x outside [0, 1] or a value that is not finite
+    unsigned blocks_done;
+};
+
+// The per-cell passes before and after a trace, for one solve.
+struct FieldJob {
+    const double* nh = nullptr;
+    const double* x = nullptr;
+    void* kap = nullptr;             // float or double
+    double* gamma = nullptr;
+    double* gamma_out = nullptr;     // Gamma's copy (null: none)
+    double* heat = nullptr;          // null: none
+    int64_t ncell = 0;
+    double sdx = 0, n_th = 0;
+    double e_heat = 0, vol = 0;
+    const FieldCheck* chk = nullptr; // given: n_th from there
+    DevStats* st = nullptr;
+    uint32_t block0 = 0;
 };
 
 enum : unsigned {
@@ -165,18 +188,22 @@ void launch_geom_fill64(long long rq, int l, const int4* dirs, long long npix, i
                         unsigned* err, cudaStream_t s);
 
 // fields.cu
-int launch_validate_fields(const double* nh, const double* x, int64_t ncell, DevStats* st, cudaStream_t s);
-int launch_prepare_kappa_f64(const double* nh, const double* x, int64_t ncell, double sdx, double n_th,
-                              double* kap, cudaStream_t s);
-int launch_prepare_kappa_f32(const double* nh, const double* x, int64_t ncell, double sdx, double n_th,
-                              float* kap, cudaStream_t s);
-int launch_finalize(const double* gamma, const double* nh, const double* x, int64_t ncell, double e_heat,
-                     double vol, double* heat, DevStats* st, cudaStream_t s);
-int launch_chem_update(const double* nh, const double* x0, double* xavg, double* xend, const double* gamma,
-                        int64_t ncell, double dt, double alpha_B, double C_H, double clump, DevStats* st,
-                        cudaStream_t s);
-int launch_sum_x(const double* x, int64_t ncell, DevStats* st, cudaStream_t s);
-int launch_mean_nh(const double* nh, int64_t ncell, double* out, cudaStream_t s);
+// New fields: invalid values counted, n_H (and x, if want_x) summed into *chk (zeroed by the caller), and
+// copied where nh_out and x_out are given.
+int launch_check_fields(const double* nh, const double* x, int64_t ncell, double* nh_out, double* x_out, bool want_x,
+                        FieldCheck* chk, cudaStream_t s);
+// kappa, and Gamma cleared.
+int launch_prepare_kappa(const FieldJob& j, bool fp32, cudaStream_t s);
+// Heating, deposited photons and the results.
+int launch_finalize(const FieldJob& j, cudaStream_t s);
+// The two over many jobs in one launch: jobs[i].block0 counts field_blocks() of the jobs before it,
+// jobs[njobs].block0 = blocks.
+uint32_t field_blocks(int64_t ncell);
+int launch_prepare_many(const FieldJob* jobs, int njobs, uint32_t blocks, bool fp32, cudaStream_t s);
+int launch_finalize_many(const FieldJob* jobs, int njobs, uint32_t blocks, cudaStream_t s);
+int launch_chem_update(const double* nh, const double* x0, const double* xavg, double* xnew, double* xend,
+                       const double* gamma, int64_t ncell, double dt, double alpha_B, double C_H, double clump,
+                       DevStats* st, cudaStream_t s);
 
 // Small device-to-host readbacks (statistics, counters), written by one kernel straight into mapped
 // pinned host memory: unlike copies they do not queue on the copy engines behind large transfers
