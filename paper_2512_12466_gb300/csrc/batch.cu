@@ -283,11 +283,11 @@ int enqueue_chunk(rt_batch* b, size_t i, int64_t first, int64_t count, int k, in
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)b->sm_count * 8));
         const bool table = tables && b->geo_ok[l];
         if constexpr (sizeof(R) == 8) {
-            if (table) launch_march_table_f64(a, b->geo[l], grid, 256, s);
-            else launch_march_f64(a, grid, 256, s);
+            if (table) launch_march_table_f64(a, b->geo[l], grid, s);
+            else launch_march_f64(a, grid, s);
         } else {
-            if (table) launch_march_table_f32(a, b->geo[l], grid, 256, s);
-            else launch_march_f32(a, grid, 256, s);
+            if (table) launch_march_table_f32(a, b->geo[l], grid, s);
+            else launch_march_f32(a, grid, s);
         }
         B_CUDA(b, cudaGetLastError(), "march launch");
         b->launches += 1;

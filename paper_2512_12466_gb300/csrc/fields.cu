@@ -211,11 +211,13 @@ __device__ __forceinline__ void finalize_cells(const FieldJob& J, const int64_t 
 template <class R>
 __global__ void __launch_bounds__(kBlock) prepare_kappa_kernel(const FieldJob J)
 {
+    if (J.valid && blockIdx.x == 0 && threadIdx.x == 0 && J.valid->bad) atomicAdd(&J.st->bad_input, J.valid->bad);
     prepare_cells<R>(J, blockIdx.x, gridDim.x);
 }
 
 __global__ void __launch_bounds__(kBlock) finalize_kernel(const FieldJob J)
 {
+    if (J.valid && J.st->bad_input) return;
     finalize_cells(J, blockIdx.x, gridDim.x);
 }
 

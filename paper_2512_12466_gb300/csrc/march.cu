@@ -1620,7 +1620,18 @@ __device__ __forceinline__ void flush_tally(Tally& T, unsigned mask, DevStats* c
             const unsigned sec = __reduce_add_sync(grp, T.sec);
             unsigned long long hash = 0ULL;
             double ab = 0.0, ep = 0.0, dp = 0.0;
-            for (unsigned g = grp; g; g &= g - 1) {
+            if (grp == 0xffffffffu) {           // the whole warp: a tree (an FP64 instruction is 64 cycles)
+                hash = T.hash;
+                ab = T.abs;
+                ep = T.escph;
+                dp = T.dropph;
+                for (int o = 16; o > 0; o >>= 1) {
+                    hash += __shfl_xor_sync(grp, hash, o);
+                    ab += __shfl_xor_sync(grp, ab, o);
+                    ep += __shfl_xor_sync(grp, ep, o);
+                    dp += __shfl_xor_sync(grp, dp, o);
+                }
+            } else for (unsigned g = grp; g; g &= g - 1) {
                 const int b = __ffs(g) - 1;
                 hash += __shfl_sync(grp, T.hash, b);
                 ab += __shfl_sync(grp, T.abs, b);
@@ -1647,6 +1658,58 @@ __device__ __forceinline__ void flush_tally(Tally& T, unsigned mask, DevStats* c
     }
 }
 
+// The tallies of a block of kBlock threads, all of one solve, summed and added to its statistics: one
+// atomic per block and counter, and none from a block without rays. The three photon sums fold in shared
+// memory, 26 FP64 warp instructions a block; one warp's sums lane after lane took 96, so that a full grid
+// spent 75 us of FP64 pipe on them, whatever it had marched. ph: 3 kLevelBlock doubles of shared memory
+// that no thread reads any more once every thread has arrived here.
+constexpr int kLevelBlock = 256;
+
+template <bool kHash>
+__device__ __forceinline__ void flush_block(const Tally& T, DevStats* st, const int l, double* const ph)
+{
+    constexpr int kWarps = kLevelBlock / 32, kCounts = 7;
+    __shared__ unsigned cnt[kWarps][kCounts];
+    const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+    if (!__syncthreads_or(T.rays != 0u)) return;
+    const unsigned mine[kCounts] = {T.rays, T.split, T.esc, T.dtau, T.dlev, T.seg, T.sec};
+#pragma unroll
+    for (int k = 0; k < kCounts; ++k) {
+        const unsigned v = __reduce_add_sync(0xffffffffu, mine[k]);
+        if (lane == 0) cnt[w][k] = v;
+    }
+    ph[t] = T.abs;
+    ph[kLevelBlock + t] = T.escph;
+    ph[2 * kLevelBlock + t] = T.dropph;
+    for (int half = kLevelBlock / 2; half > 0; half >>= 1) {
+        __syncthreads();
+        for (int i = t; i < 3 * half; i += kLevelBlock) {
+            double* const p = ph + (i / half) * kLevelBlock + i % half;
+            *p += p[half];
+        }
+    }
+    __syncthreads();
+    if (t < kCounts) {
+        unsigned long long* const to[kCounts] = {&st->rays[l], &st->splits[l], &st->escaped[l], &st->dropped_tau[l],
+                                                 &st->dropped_level[l], &st->segments[l], &st->secondary[l]};
+        unsigned long long v = 0;
+        for (int q = 0; q < kWarps; ++q) v += cnt[q][t];
+        unsigned long long* dst = to[0];
+#pragma unroll
+        for (int k = 1; k < kCounts; ++k) dst = t == k ? to[k] : dst;
+        if (v) atomicAdd(dst, v);
+    } else if (t >= 32 && t < 35) {
+        const double v = ph[(t - 32) * kLevelBlock];
+        double* const dst = t == 32 ? &st->absorbed : (t == 33 ? &st->escaped_ph : &st->dropped_ph);
+        if (__double_as_longlong(v) << 1) atomicAdd(dst, v);
+    }
+    if constexpr (kHash) {
+        unsigned long long h = T.hash;
+        for (int o = 16; o > 0; o >>= 1) h += __shfl_xor_sync(0xffffffffu, h, o);
+        if (lane == 0 && h) atomicAdd(&st->visit_hash, h);
+    }
+}
+
 // Resident blocks of 256 threads per SM the march kernels are compiled for:
 // the FP32 march fits 80 registers without spilling, so three blocks (24
 // warps) hide more of its dependency latency than two; the FP64 march is held
@@ -1656,10 +1719,29 @@ struct MarchOccupancy {
     static constexpr int blocks = sizeof(R) == 4 ? 3 : 2;
 };
 
+// A level that was launched before the previous one had ended waits here for it (at once otherwise),
+// and lets the next one be launched: its blocks then start in the tail of this launch.
+__device__ __forceinline__ void march_grid_wait()
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// End of a launch's child range: as given, or bounded by what the device counted.
+template <class R>
+__device__ __forceinline__ long long launch_end(const MarchArgs<R>& A)
+{
+    long long c1 = A.c1;
+    if (A.in_count) c1 = min(c1, (long long)A.c0 + 4LL * (long long)*A.in_count);
+    if (A.src_count) c1 = min(c1, 12LL * *A.src_count);
+    if (A.bad_input && *A.bad_input) c1 = A.c0;
+    return c1;
+}
+
 // One level (or one slice of it) of one solve: thread j marches child j.
 // kHash: compiled with the visit hash (only launched when it is asked for).
 template <class R, bool kHash, bool kFreq>
-__global__ void __launch_bounds__(256, MarchOccupancy<R>::blocks) march_kernel(const MarchArgs<R> A)
+__global__ void __launch_bounds__(kLevelBlock, MarchOccupancy<R>::blocks) march_kernel(const MarchArgs<R> A)
 {
     const int l = A.level;
     const int lane = threadIdx.x & 31;
@@ -1677,8 +1759,8 @@ __global__ void __launch_bounds__(256, MarchOccupancy<R>::blocks) march_kernel(c
     V.src_off = 0;
     V.rs = A.rs;
     V.spec = A.spec;
-    // children of this launch: as given, or bounded by the parents the previous level counted
-    const long long c1 = A.in_count ? min((long long)A.c1, (long long)A.c0 + 4LL * (long long)*A.in_count) : (long long)A.c1;
+    march_grid_wait();
+    const long long c1 = launch_end(A);
     Tally T;
     T.clear();
     for (long long base = A.c0 + gwarp * 32; base < c1; base += nwarp * 32) {
@@ -1695,8 +1777,8 @@ __global__ void __launch_bounds__(256, MarchOccupancy<R>::blocks) march_kernel(c
         }
         append_split<R>(split, si, pix, oP, otau, ocP, octau, A.out, A.out_count, &A.st->err);
     }
-    DevStats* st = A.st;
-    flush_tally(T, 0xffffffffu, &st, l);
+    __shared__ double ph[3 * kLevelBlock];
+    flush_block<kHash>(T, A.st, l, ph);
 }
 
 // One level (or one slice of it) of one solve, geometry from the level's table (kFreq: Eq. 1 over
@@ -1709,7 +1791,7 @@ struct TableOccupancy {
 };
 
 template <class R, bool kHash, bool kFreq>
-__global__ void __launch_bounds__(256, TableOccupancy<R>::blocks) march_table_kernel(const MarchArgs<R> A, const GeomLevel GL)
+__global__ void __launch_bounds__(kLevelBlock, TableOccupancy<R>::blocks) march_table_kernel(const MarchArgs<R> A, const GeomLevel GL)
 {
     const int l = A.level;
     const int lane = threadIdx.x & 31;
@@ -1727,8 +1809,6 @@ __global__ void __launch_bounds__(256, TableOccupancy<R>::blocks) march_table_ke
     V.src_off = 0;
     V.rs = A.rs;
     V.spec = A.spec;
-    // children of this launch: as given, or bounded by the parents the previous level counted
-    const long long c1 = A.in_count ? min((long long)A.c1, (long long)A.c0 + 4LL * (long long)*A.in_count) : (long long)A.c1;
     Tally T;
     T.clear();
     // FP64 march in double-float arithmetic; gray: the Eq. 1 rate table in shared memory (two float4
@@ -1742,6 +1822,8 @@ __global__ void __launch_bounds__(256, TableOccupancy<R>::blocks) march_table_ke
         }
         __syncthreads();
     }
+    march_grid_wait();
+    const long long c1 = launch_end(A);
     for (long long base = A.c0 + gwarp * 32; base < c1; base += nwarp * 32) {
         const long long j = base + lane;
         bool split = false;
@@ -1761,8 +1843,12 @@ __global__ void __launch_bounds__(256, TableOccupancy<R>::blocks) march_table_ke
         }
         append_split<R>(split, si, pix, oP, otau, ocP, octau, A.out, A.out_count, &A.st->err);
     }
-    DevStats* st = A.st;
-    flush_tally(T, 0xffffffffu, &st, l);
+    if constexpr (kDf && !kFreq) {                // the rate table's place: a third smaller footprint
+        flush_block<kHash>(T, A.st, l, reinterpret_cast<double*>(rtab));
+    } else {
+        __shared__ double ph[3 * kLevelBlock];
+        flush_block<kHash>(T, A.st, l, ph);
+    }
 }
 
 // All solves of a batch in one cooperative launch. Every block runs the same
@@ -1887,52 +1973,61 @@ __global__ void __launch_bounds__(256, (kTable && kSingle) ? TableOccupancy<R>::
 
 }  // namespace
 
+// One march launch; a.early: as soon as the previous launch of the stream lets it (it waits in
+// march_grid_wait for that launch's results).
+template <class... P, class... Args>
+static void launch_level(void (*kernel)(P...), bool early, int grid, cudaStream_t s, const Args&... args)
+{
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3((unsigned)grid);
+    c.blockDim = dim3((unsigned)kLevelBlock);
+    c.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = at;
+    c.numAttrs = early ? 1 : 0;
+    cudaLaunchKernelEx(&c, kernel, args...);
+}
+
 template <class R>
-static int launch_march_impl(const MarchArgs<R>& a, int grid, int block, cudaStream_t s)
+static int launch_march_impl(const MarchArgs<R>& a, int grid, cudaStream_t s)
 {
     const bool freq = a.spec.lin_a != nullptr;
-    if (a.hash) {
-        if (freq) march_kernel<R, true, true><<<grid, block, 0, s>>>(a);
-        else march_kernel<R, true, false><<<grid, block, 0, s>>>(a);
-    } else {
-        if (freq) march_kernel<R, false, true><<<grid, block, 0, s>>>(a);
-        else march_kernel<R, false, false><<<grid, block, 0, s>>>(a);
-    }
+    auto* k = a.hash ? (freq ? march_kernel<R, true, true> : march_kernel<R, true, false>)
+                     : (freq ? march_kernel<R, false, true> : march_kernel<R, false, false>);
+    launch_level(k, a.early, grid, s, a);
     return 1;
 }
 
-int launch_march_f64(const MarchArgs<double>& a, int grid, int block, cudaStream_t s)
+int launch_march_f64(const MarchArgs<double>& a, int grid, cudaStream_t s)
 {
-    return launch_march_impl<double>(a, grid, block, s);
+    return launch_march_impl<double>(a, grid, s);
 }
 
-int launch_march_f32(const MarchArgs<float>& a, int grid, int block, cudaStream_t s)
+int launch_march_f32(const MarchArgs<float>& a, int grid, cudaStream_t s)
 {
-    return launch_march_impl<float>(a, grid, block, s);
+    return launch_march_impl<float>(a, grid, s);
 }
 
-int launch_march_table_f32(const MarchArgs<float>& a, const GeomLevel& g, int grid, int block, cudaStream_t s)
+template <class R>
+static int launch_march_table_impl(const MarchArgs<R>& a, const GeomLevel& g, int grid, cudaStream_t s)
 {
-    if (a.spec.lin_a) {
-        if (a.hash) march_table_kernel<float, true, true><<<grid, block, 0, s>>>(a, g);
-        else march_table_kernel<float, false, true><<<grid, block, 0, s>>>(a, g);
-    } else {
-        if (a.hash) march_table_kernel<float, true, false><<<grid, block, 0, s>>>(a, g);
-        else march_table_kernel<float, false, false><<<grid, block, 0, s>>>(a, g);
-    }
+    const bool freq = a.spec.lin_a != nullptr;
+    auto* k = a.hash ? (freq ? march_table_kernel<R, true, true> : march_table_kernel<R, true, false>)
+                     : (freq ? march_table_kernel<R, false, true> : march_table_kernel<R, false, false>);
+    launch_level(k, a.early, grid, s, a, g);
     return 1;
 }
 
-int launch_march_table_f64(const MarchArgs<double>& a, const GeomLevel& g, int grid, int block, cudaStream_t s)
+int launch_march_table_f32(const MarchArgs<float>& a, const GeomLevel& g, int grid, cudaStream_t s)
 {
-    if (a.spec.lin_a) {
-        if (a.hash) march_table_kernel<double, true, true><<<grid, block, 0, s>>>(a, g);
-        else march_table_kernel<double, false, true><<<grid, block, 0, s>>>(a, g);
-    } else {
-        if (a.hash) march_table_kernel<double, true, false><<<grid, block, 0, s>>>(a, g);
-        else march_table_kernel<double, false, false><<<grid, block, 0, s>>>(a, g);
-    }
-    return 1;
+    return launch_march_table_impl<float>(a, g, grid, s);
+}
+
+int launch_march_table_f64(const MarchArgs<double>& a, const GeomLevel& g, int grid, cudaStream_t s)
+{
+    return launch_march_table_impl<double>(a, g, grid, s);
 }
 
 void launch_geom_count(long long rq, int l, const int4* dirs, long long npix, int n_cover, long long rs,

@@ -177,8 +177,8 @@ int na_level(Ctx& c, int level, int64_t nparents)
         a.hash = c.hash;
         a.st = c.st;
         const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((c1 - c0 + 255) / 256, 152 * 8));
-        if constexpr (sizeof(R) == 8) c.launches += launch_march_f64(a, grid, 256, c.s);
-        else c.launches += launch_march_f32(a, grid, 256, c.s);
+        if constexpr (sizeof(R) == 8) c.launches += launch_march_f64(a, grid, c.s);
+        else c.launches += launch_march_f32(a, grid, c.s);
         if (cudaGetLastError() != cudaSuccess) return set_error(RT_ECUDA, "rt_step_noalloc: march launch failed");
         unsigned long long next = 0;
         unsigned err = 0;

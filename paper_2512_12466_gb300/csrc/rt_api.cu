@@ -39,6 +39,12 @@ thread_local std::string g_create_error;
 // followed by its whole sub-tree, which bounds every ray buffer to this many
 // records.
 constexpr int64_t kMaxChildrenPerLaunch = int64_t(1) << 27;
+// Levels that can hold at most this many rays are launched one behind the other without the host
+// knowing their size: each launch takes it from the count the level before it left on the device. The
+// bound is what the next level's ray buffer is sized for (24 bytes a record, 25 MB). A host round trip
+// costs 15-25 us, which for a level of a million rays is below a tenth of its march; four levels launched
+// in vain (an opaque box whose rays end at level 0) cost 2.5 us each.
+constexpr int64_t kChainChildren = int64_t(1) << 20;
 constexpr int kMarchBlock = 256;
 constexpr int kMarchBlocksPerSm = 12;
 constexpr char kBadInput[] = "invalid field or source values (n_H < 0, x outside [0,1], non-finite, bad source)";
@@ -620,85 +626,102 @@ int ensure_rays(rt_handle* h, int level, int64_t need)
     return RT_OK;
 }
 
-// March all rays of `level` whose parents are the first n records of the
-// level's buffer (level 0: the emitted sources), then recurse into the
-// next level, one slice of children at a time.
+// One march launch: children [c0, c1) of `level`, or as many of them as the device counted (counted).
 template <class R>
-int run_level(rt_handle* h, int level, int64_t nparents)
+int launch_level(rt_handle* h, int level, int64_t c0, int64_t c1, bool counted, bool early)
 {
     char range[32];
     std::snprintf(range, sizeof(range), "march level %d", level);
     NvtxRange nvtx(range);
-    const int64_t total = level == 0 ? 12 * h->n_emit : 4 * nparents;
+    // rays of the deepest level end before their split sphere or at level_max
+    const bool can_split = level < h->table_level;
+    if (can_split) {
+        const int rc = ensure_rays<R>(h, level + 1, c1 - c0);
+        if (rc) return rc;
+    }
+    MarchArgs<R> a;
+    a.level = level;
+    a.n = h->cfg.n;
+    a.c0 = c0;
+    a.c1 = c1;
+    a.in_count = counted && level > 0 ? h->d_count + level : nullptr;
+    if (level == 0) {
+        a.src_count = h->n_emit < 0 ? h->sw.count : nullptr;
+        a.bad_input = &h->d_st->bad_input;
+    }
+    a.early = early;
+    a.dirs = h->dirs + healpix_level_offset(level);
+    a.src = h->d_emit;
+    a.in = ray_view<R>(h->rays[level]);
+    a.out = can_split ? ray_view<R>(h->rays[level + 1]) : RayBuf<R>();
+    a.out_count = h->d_count + level + 1;
+    a.kap = static_cast<const R*>(h->d_kap);
+    a.gamma = h->d_gamma;
+    a.rq = h->rq;
+    a.level_max = h->level_max;
+    a.tau_max = (R)h->cfg.tau_max;
+    a.overlap_mode = h->cfg.overlap_mode;
+    a.hash = (h->cfg.flags & RT_FLAG_VISIT_HASH) ? 1 : 0;
+    a.rs = h->rs;
+    if constexpr (sizeof(R) == 8) a.spec = h->spec_d;
+    else a.spec = h->spec_f;
+    a.st = h->d_st;
+    const int64_t warps = (c1 - c0 + 31) / 32;
+    const int64_t want = (warps + kMarchBlock / 32 - 1) / (kMarchBlock / 32);
+    // grid-stride blocks of equal share: 12 per SM is a whole number of waves for the march
+    // kernels' 2, 3 and 4 resident blocks per SM, so no last wave runs an SM part-empty
+    const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)h->sm_count * kMarchBlocksPerSm));
+    // the level's geometry table for this precision (built once per device)
+    GeomLevel gl;
+    const bool table = !(h->cfg.flags & RT_FLAG_NO_GEOMETRY_TABLE) &&
+                       geometry_level(h->device, h->rq, level, h->cfg.n, h->rs, a.dirs, h->stream, sizeof(R) == 8, &gl);
+    if constexpr (sizeof(R) == 8) {
+        if (table) launch_march_table_f64(a, gl, grid, h->stream);
+        else launch_march_f64(a, grid, h->stream);
+    } else {
+        if (table) launch_march_table_f32(a, gl, grid, h->stream);
+        else launch_march_f32(a, grid, h->stream);
+    }
+    RT_LAUNCHED(h, "march launch");
+    h->launches++;
+    h->march_launches++;
+    if (table) h->table_levels |= int64_t(1) << level;
+    return RT_OK;
+}
+
+// March `total` rays of `level` and all that follow from them, one slice of children at a time.
+// A slice's next levels are enqueued behind it while their bound (every ray splits) stays within
+// kChainChildren; the host reads the count of the level after those, if there is one, and goes on from
+// there. counted: `total` is a bound itself (level 0, with the catalog's size on the device).
+template <class R>
+int run_levels(rt_handle* h, int level, int64_t total, bool counted)
+{
     if (total <= 0) return RT_OK;
     if (level > h->table_level || level > kMaxLevel)
         return fail(h, RT_EDEVICE, "ray level beyond the direction table");
-    const bool can_split = level + 1 <= h->level_max;
     for (int64_t c0 = 0; c0 < total; c0 += kMaxChildrenPerLaunch) {
         const int64_t c1 = std::min(total, c0 + kMaxChildrenPerLaunch);
-        if (can_split) {
-            int rc = ensure_rays<R>(h, level + 1, c1 - c0);
+        RT_CUDA(h, cudaMemsetAsync(h->d_count + level + 1, 0, sizeof(unsigned long long) * (size_t)(RT_MAX_LEVELS - level),
+                                   h->stream), "counters");
+        int l = level;
+        int64_t bound = c1 - c0;
+        int rc = launch_level<R>(h, l, c0, c1, counted, false);
+        if (rc) return rc;
+        while (l < h->table_level && 4 * bound <= kChainChildren) {
+            ++l;
+            bound *= 4;
+            rc = launch_level<R>(h, l, 0, bound, true, true);
             if (rc) return rc;
         }
-        RT_CUDA(h, cudaMemsetAsync(h->d_count + level + 1, 0, sizeof(unsigned long long), h->stream), "counter");
-        MarchArgs<R> a;
-        a.level = level;
-        a.n = h->cfg.n;
-        a.c0 = c0;
-        a.c1 = c1;
-        a.dirs = h->dirs + healpix_level_offset(level);
-        a.src = h->d_emit;
-        a.in = ray_view<R>(h->rays[level]);
-        a.out = can_split ? ray_view<R>(h->rays[level + 1]) : RayBuf<R>();
-        a.out_count = h->d_count + level + 1;
-        a.kap = static_cast<const R*>(h->d_kap);
-        a.gamma = h->d_gamma;
-        a.rq = h->rq;
-        a.level_max = h->level_max;
-        a.tau_max = (R)h->cfg.tau_max;
-        a.overlap_mode = h->cfg.overlap_mode;
-        a.hash = (h->cfg.flags & RT_FLAG_VISIT_HASH) ? 1 : 0;
-        a.rs = h->rs;
-        if constexpr (sizeof(R) == 8) a.spec = h->spec_d;
-        else a.spec = h->spec_f;
-        a.st = h->d_st;
-        const int64_t warps = (c1 - c0 + 31) / 32;
-        const int64_t want = (warps + kMarchBlock / 32 - 1) / (kMarchBlock / 32);
-        // grid-stride blocks of equal share: 12 per SM is a whole number of waves for the march
-        // kernels' 2, 3 and 4 resident blocks per SM, so no last wave runs an SM part-empty
-        const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)h->sm_count * kMarchBlocksPerSm));
-        // the level's geometry table for this precision (built once per device, outside the timed launch)
-        GeomLevel gl;
-        const bool table = !(h->cfg.flags & RT_FLAG_NO_GEOMETRY_TABLE) &&
-                           geometry_level(h->device, h->rq, level, h->cfg.n, h->rs, a.dirs, h->stream, sizeof(R) == 8,
-                                          &gl);
-        RT_CUDA(h, cudaEventRecord(h->ev[4], h->stream), "event");
-        if constexpr (sizeof(R) == 8) {
-            if (table) launch_march_table_f64(a, gl, grid, kMarchBlock, h->stream);
-            else launch_march_f64(a, grid, kMarchBlock, h->stream);
-        } else {
-            if (table) launch_march_table_f32(a, gl, grid, kMarchBlock, h->stream);
-            else launch_march_f32(a, grid, kMarchBlock, h->stream);
-        }
-        RT_LAUNCHED(h, "march launch");
-        RT_CUDA(h, cudaEventRecord(h->ev[5], h->stream), "event");
-        h->launches++;
-        h->march_launches++;
-        if (table) h->table_levels |= int64_t(1) << level;
-        RT_CUDA(h, cudaMemcpyAsync(h->h_count + level + 1, h->d_count + level + 1, sizeof(unsigned long long),
+        if (l == h->table_level) continue;
+        RT_CUDA(h, cudaMemcpyAsync(h->h_count + l + 1, h->d_count + l + 1, sizeof(unsigned long long),
                                    cudaMemcpyDeviceToHost, h->stream), "counter read");
         RT_CUDA(h, cudaMemcpyAsync(h->h_i32, &h->d_st->err, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream),
                 "error read");
         RT_CUDA(h, cudaStreamSynchronize(h->stream), "march");
         if (h->h_i32[0]) return fail(h, RT_EDEVICE, "march kernel reported an internal error");
-        float ms = 0.f;
-        RT_CUDA(h, cudaEventElapsedTime(&ms, h->ev[4], h->ev[5]), "event");
-        h->ms_march += ms;
-        const int64_t next = (int64_t)h->h_count[level + 1];
-        if (next > 0) {
-            int rc = run_level<R>(h, level + 1, next);
-            if (rc) return rc;
-        }
+        rc = run_levels<R>(h, l + 1, 4 * (int64_t)h->h_count[l + 1], false);
+        if (rc) return rc;
     }
     return RT_OK;
 }
@@ -745,18 +768,23 @@ bool direct_access(const rt_handle* h, const void* p)
     return a.type == cudaMemoryTypeDevice && a.device == h->device;
 }
 
-int trace(rt_handle* h, const double* xuse)
+// first: the step's first trace, with the statistics as rt_step cleared them.
+int trace(rt_handle* h, const double* xuse, bool first)
 {
     // per-trace part of the statistics: per-level counters, hash and ledger
-    RT_CUDA(h, cudaMemsetAsync(h->d_st, 0, offsetof(DevStats, deposited), h->stream), "stats clear");
-    launch_prepare_kappa(field_job(h, xuse), h->cfg.precision == RT_FP32, h->stream);
+    if (!first) RT_CUDA(h, cudaMemsetAsync(h->d_st, 0, offsetof(DevStats, deposited), h->stream), "stats clear");
+    FieldJob job = field_job(h, xuse);
+    job.valid = first ? h->d_chk : nullptr;
+    launch_prepare_kappa(job, h->cfg.precision == RT_FP32, h->stream);
     RT_LAUNCHED(h, "kappa launch");
     h->launches++;
     h->march_launches = 0;
     h->table_levels = 0;
-    h->ms_march = 0.0;
     RT_CUDA(h, cudaEventRecord(h->ev[1], h->stream), "event");
-    int rc = h->cfg.precision == RT_FP32 ? run_level<float>(h, 0, 0) : run_level<double>(h, 0, 0);
+    const bool counted = h->n_emit < 0;
+    const int64_t total = 12 * (counted ? h->nsrc : h->n_emit);
+    const int rc = h->cfg.precision == RT_FP32 ? run_levels<float>(h, 0, total, counted)
+                                               : run_levels<double>(h, 0, total, counted);
     if (rc) return rc;
     RT_CUDA(h, cudaEventRecord(h->ev[2], h->stream), "event");
     return RT_OK;
@@ -765,7 +793,7 @@ int trace(rt_handle* h, const double* xuse)
 // Sec. 2.8 source stage of a step: validation of device-resident inputs,
 // dedup + sort, the n_th default, Alg. 3 merging when on, and the emitted
 // catalog (h->d_emit, h->n_emit). Leaves the field check in h->h_chk.
-int prepare_sources(rt_handle* h, bool* merged_out, int64_t* n_dedup_out)
+int prepare_sources(rt_handle* h, bool wait, bool* merged_out, int64_t* n_dedup_out)
 {
     NvtxRange nvtx("source stage (dedup, sort, Alg. 3)");
     cudaStream_t s = h->stream;
@@ -782,6 +810,12 @@ int prepare_sources(rt_handle* h, bool* merged_out, int64_t* n_dedup_out)
     // ---- sources: dedup + sort (Sec. 2.8)
     h->launches += launch_dedup_sort(h->sw, h->nsrc, h->cfg.n, s);
     RT_LAUNCHED(h, "source launch");
+    if (!wait && h->cfg.merge_mode == RT_MERGE_OFF) {
+        h->launches += launch_build_emit_dev(h->sw, h->nsrc, h->s_over_dx2, h->d_emit, h->d_st, s);
+        RT_LAUNCHED(h, "emit launch");
+        h->n_emit = h->nsrc > 0 ? -1 : 0;
+        return RT_OK;
+    }
     RT_CUDA(h, cudaMemcpyAsync(h->h_st, h->d_st, sizeof(DevStats), cudaMemcpyDeviceToHost, s), "stats read");
     if (h->nsrc > 0)
         RT_CUDA(h, cudaMemcpyAsync(h->h_i32, h->sw.count, sizeof(int32_t), cudaMemcpyDeviceToHost, s), "count read");
@@ -907,7 +941,7 @@ int handle_prepare_sources(rt_handle* h)
     RT_CUDA(h, cudaMemsetAsync(h->d_st, 0, sizeof(DevStats), h->stream), "stats clear");
     bool merged = false;
     int64_t nd = 0;
-    const int rc = prepare_sources(h, &merged, &nd);
+    const int rc = prepare_sources(h, true, &merged, &nd);
     if (rc) return rc;
     RT_CUDA(h, cudaMemcpyAsync(h->h_st, h->d_st, sizeof(DevStats), cudaMemcpyDeviceToHost, h->stream), "stats");
     RT_CUDA(h, cudaStreamSynchronize(h->stream), "source stage");
@@ -1325,6 +1359,14 @@ int rt_get_x(rt_handle* h, double* x_out, int where)
     return RT_OK;
 }
 
+// Invalid fields or sources found on the device: nothing was traced and no result written.
+static int reject(rt_handle* h)
+{
+    h->n_emit = 0;
+    h->catalog_valid = false;
+    return fail(h, RT_EINVAL, kBadInput);
+}
+
 int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int where, rt_stats* st)
 {
     NvtxRange nvtx("rt_step");
@@ -1343,10 +1385,10 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
     bool merged = false;
     int64_t n_dedup = 0;
     {
-        const int rc = prepare_sources(h, &merged, &n_dedup);
+        const int rc = prepare_sources(h, false, &merged, &n_dedup);
         if (rc) return rc;
     }
-    const int64_t m = h->n_emit;
+    h->ms_march = 0.0;
 
     // ---- trace, optionally iterated with the C2-Ray update (Sec. 2.4)
     int iters = 0;
@@ -1358,17 +1400,26 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
         // one the last trace used stays, for the heating
         double* xnew = h->d_xavg;
         for (;;) {
-            int rc = trace(h, xuse);
+            int rc = trace(h, xuse, iters == 0);
             if (rc) return rc;
             ++iters;
             RT_CUDA(h, cudaMemsetAsync(&h->d_st->maxdiff, 0, sizeof(double), s), "clear");
             h->launches += launch_chem_update(h->d_nh, h->d_x, xuse, xnew, h->d_xend, h->d_gamma, h->ncell, dt_s,
                                               h->cfg.alpha_B, h->cfg.C_H, h->cfg.clumping, h->d_st, s);
             RT_LAUNCHED(h, "chemistry launch");
-            RT_CUDA(h, cudaMemcpyAsync(h->h_f64 + 2, &h->d_st->maxdiff, sizeof(double), cudaMemcpyDeviceToHost, s),
+            // the residual, and the error words beside it
+            static_assert(offsetof(DevStats, bad_input) == offsetof(DevStats, maxdiff) + 12, "read together");
+            RT_CUDA(h, cudaMemcpyAsync(h->h_f64 + 2, &h->d_st->maxdiff, 2 * sizeof(double), cudaMemcpyDeviceToHost, s),
                     "residual read");
             RT_CUDA(h, cudaStreamSynchronize(s), "chemistry");
             resid = h->h_f64[2];
+            unsigned words[2];
+            std::memcpy(words, h->h_f64 + 3, sizeof(words));
+            if (words[1]) return reject(h);
+            if (words[0]) return fail(h, RT_EDEVICE, "march kernel reported an internal error");
+            float ms = 0.f;
+            RT_CUDA(h, cudaEventElapsedTime(&ms, h->ev[1], h->ev[2]), "event");
+            h->ms_march = ms;
             if (resid < h->cfg.chem_tol || iters >= maxit) break;
             xuse = xnew;
             xnew = xnew == h->d_xavg ? h->d_heat : h->d_xavg;
@@ -1376,7 +1427,7 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
         // heating uses the <x> the last trace used; it may be d_heat, which then takes the other's place
         if (xuse == h->d_heat) std::swap(h->d_xavg, h->d_heat);
     } else {
-        int rc = trace(h, h->d_x);
+        int rc = trace(h, h->d_x, true);
         if (rc) return rc;
         iters = 1;
     }
@@ -1390,6 +1441,7 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
     const bool gamma_direct = gamma_out && where == RT_DEVICE && apart && direct_access(h, gamma_out);
     const bool heat_direct = heat_out && where == RT_DEVICE && apart && direct_access(h, heat_out);
     FieldJob job = field_job(h, xuse);
+    job.valid = h->d_chk;
     job.gamma_out = gamma_direct ? gamma_out : nullptr;
     job.heat = heat_direct ? heat_out : (heat_out ? h->d_heat : nullptr);
     h->launches += launch_finalize(job, s);
@@ -1399,19 +1451,31 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
         h->fields_checked = false;
     }
     const cudaMemcpyKind k = where == RT_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
+    if ((gamma_out && !gamma_direct) || (heat_out && !heat_direct)) {
+        // nothing is copied over the caller's data before the inputs are known to be valid
+        RT_CUDA(h, cudaMemcpyAsync(h->h_i32, &h->d_st->bad_input, sizeof(unsigned), cudaMemcpyDeviceToHost, s), "input check");
+        RT_CUDA(h, cudaStreamSynchronize(s), "step");
+        if (h->h_i32[0]) return reject(h);
+    }
     if (gamma_out && !gamma_direct) RT_CUDA(h, cudaMemcpyAsync(gamma_out, h->d_gamma, fb, k, s), "gamma copy");
     if (heat_out && !heat_direct) RT_CUDA(h, cudaMemcpyAsync(heat_out, h->d_heat, fb, k, s), "heat copy");
     RT_CUDA(h, cudaEventRecord(h->ev[3], s), "event");
     RT_CUDA(h, cudaMemcpyAsync(h->h_st, h->d_st, sizeof(DevStats), cudaMemcpyDeviceToHost, s), "stats read");
     RT_CUDA(h, cudaStreamSynchronize(s), "step");
+    if (h->h_st->bad_input) return reject(h);
     if (h->h_st->err) return fail(h, RT_EDEVICE, "a kernel reported an internal error");
+    if (h->n_emit < 0) {                      // counted on the device, without merging
+        h->n_emit = h->h_st->n_emit;
+        n_dedup = h->n_emit;
+    }
+    h->catalog_valid = true;
 
     if (st) {
         std::memset(st, 0, sizeof(*st));
         const DevStats& d = *h->h_st;
         st->n_src_in = h->nsrc;
         st->n_src_dedup = n_dedup;
-        st->n_src_emit = m;
+        st->n_src_emit = h->n_emit;
         st->merged = merged ? 1 : 0;
         st->chem_iters = iters;
         st->level_max = h->level_max;
@@ -1437,7 +1501,7 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
         st->ms_trace = ms;
         cudaEventElapsedTime(&ms, h->ev[0], h->ev[3]);
         st->ms_step = ms;
-        st->ms_march = h->ms_march;
+        st->ms_march = h->cfg.chem_iterate ? h->ms_march : st->ms_trace;
         st->march_launches = h->march_launches;
         st->table_levels = h->table_levels;
     }

@@ -152,7 +152,9 @@ inline T* pinned_dev(const rt_handle* h, T* host)
 {
     return reinterpret_cast<T*>(h->d_pin + (reinterpret_cast<char*>(host) - static_cast<char*>(h->h_pin)));
 }
-int prepare_sources(rt_handle* h, bool* merged_out, int64_t* n_dedup_out);
+// The source stage of a step. Without merging it is only enqueued: the catalog's size then stays on the
+// device (h->n_emit is -1 until the step has ended) and invalid inputs show in DevStats::bad_input.
+int prepare_sources(rt_handle* h, bool wait, bool* merged_out, int64_t* n_dedup_out);
 int ensure_directions(int device, int level, const int4** out, std::string& err);
 // The geometry table of a level for grids of n cells, with the entries of the FP32 march (fp64
 // false) or the FP64 one, built on stream s if needed; false if the level has none for that

@@ -46,6 +46,8 @@ struct DevStats {
     double maxdiff;                  // chemistry: max |<x>_new - <x>_old| (as ordered bits)
     unsigned int err;                // RT_ERR_* bits set by kernels
     unsigned int bad_input;          // count of invalid field / source values
+    int n_emit;                      // sources traced
+    int pad_;
 };
 
 // What one pass over a handle's fields finds.
@@ -68,6 +70,8 @@ struct FieldJob {
     double sdx = 0, n_th = 0;
     double e_heat = 0, vol = 0;
     const FieldCheck* chk = nullptr; // given: n_th from there
+    const FieldCheck* valid = nullptr; // given: its invalid cells go to st->bad_input before the trace, and
+                                       // where that is not zero no result is written
     DevStats* st = nullptr;
     uint32_t block0 = 0;
 };
@@ -116,6 +120,11 @@ struct MarchArgs {
     // parents of this level counted on the device (written by the previous level's launch): the
     // launch then covers children [c0, min(c1, c0 + 4 * *in_count)); null: [c0, c1) as given
     const unsigned long long* in_count = nullptr;
+    // level 0 of a catalog counted on the device: children [c0, min(c1, 12 * *src_count)), and none at
+    // all where the inputs were found invalid (*bad_input)
+    const int32_t* src_count = nullptr;
+    const unsigned* bad_input = nullptr;
+    bool early = false;              // launched before the previous level has ended (march_grid_wait)
 };
 
 // Geometry table of one level (FP32 march): 8-byte entries, entry s of pixel p at
@@ -166,15 +175,15 @@ struct BatchArgs {
     SpecTable<R> spec;
 };
 
-// march.cu
-int launch_march_f64(const MarchArgs<double>& a, int grid, int block, cudaStream_t s);
-int launch_march_f32(const MarchArgs<float>& a, int grid, int block, cudaStream_t s);
+// march.cu (the per-level launches run blocks of 256 threads)
+int launch_march_f64(const MarchArgs<double>& a, int grid, cudaStream_t s);
+int launch_march_f32(const MarchArgs<float>& a, int grid, cudaStream_t s);
 cudaError_t launch_batch_f64(const BatchArgs<double>& a, int grid, int block, cudaStream_t s);
 cudaError_t launch_batch_f32(const BatchArgs<float>& a, int grid, int block, cudaStream_t s);
 int batch_blocks_per_sm(int precision, int block, bool table, bool single, bool freq);
 // The march of one level with its geometry from a table (FP32: g.ent; FP64: g.ent64).
-int launch_march_table_f32(const MarchArgs<float>& a, const GeomLevel& g, int grid, int block, cudaStream_t s);
-int launch_march_table_f64(const MarchArgs<double>& a, const GeomLevel& g, int grid, int block, cudaStream_t s);
+int launch_march_table_f32(const MarchArgs<float>& a, const GeomLevel& g, int grid, cudaStream_t s);
+int launch_march_table_f64(const MarchArgs<double>& a, const GeomLevel& g, int grid, cudaStream_t s);
 // Geometry-table generation for level l of directions dirs (npix pixels), for grids up to
 // n_cover: rows[b] = rows of 32-pixel block b; then the entries at row offsets row0.
 // rs: travel-distance cutoff of periodic boundaries (0: none).

@@ -511,6 +511,7 @@ __global__ void build_emit_dev_kernel(const int32_t* __restrict__ cells, const d
                                       DevStats* st)
 {
     const int64_t m = *count;
+    if (blockIdx.x == 0 && threadIdx.x == 0) st->n_emit = (int)m;
     double emitted = 0.0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m; i += (int64_t)gridDim.x * blockDim.x) {
         SrcEntry e;
