@@ -290,8 +290,7 @@ extern "C" int rt_step_noalloc(const rt_config* cfg, void* cuda_stream, const do
     if ((rc = cu(cudaMemsetAsync(c.st, 0, sizeof(DevStats), s), "rt_step_noalloc: statistics clear failed"))) return rc;
     if ((rc = cu(cudaMemsetAsync(chk, 0, sizeof(FieldCheck), s), "rt_step_noalloc: clear failed"))) return rc;
     c.launches += launch_check_fields(n_H, x_ion, ncell, nullptr, nullptr, false, chk, s);
-    c.launches += launch_validate_sources(cell_ijk, ndot, nsrc, n, c.st, s);
-    c.launches += launch_dedup_sort(w, nsrc, n, s);
+    c.launches += launch_sources(w, nsrc, n, cfg->sigma_cm2 / (dx * dx), emit, c.st, s);
     if ((rc = cu(cudaGetLastError(), "rt_step_noalloc: launch failed"))) return rc;
     unsigned bad = 0, bad_fields = 0;
     int32_t m32 = 0;
@@ -303,7 +302,6 @@ extern "C" int rt_step_noalloc(const rt_config* cfg, void* cuda_stream, const do
     if (bad || bad_fields) return set_error(RT_EINVAL, "rt_step_noalloc: invalid field or source values");
     const int64_t m = nsrc > 0 ? m32 : 0;
     c.n_emit = m;
-    c.launches += launch_build_emit(w, m, cfg->sigma_cm2 / (dx * dx), emit, c.st, s);
     FieldJob job;
     job.nh = n_H;
     job.x = x_ion;

@@ -41,10 +41,10 @@ thread_local std::string g_create_error;
 constexpr int64_t kMaxChildrenPerLaunch = int64_t(1) << 27;
 // Levels that can hold at most this many rays are launched one behind the other without the host
 // knowing their size: each launch takes it from the count the level before it left on the device. The
-// bound is what the next level's ray buffer is sized for (24 bytes a record, 25 MB). A host round trip
+// bound is what the next level's ray buffer is sized for (24 bytes a record, 50 MB). A host round trip
 // costs 15-25 us, which for a level of a million rays is below a tenth of its march; four levels launched
 // in vain (an opaque box whose rays end at level 0) cost 2.5 us each.
-constexpr int64_t kChainChildren = int64_t(1) << 20;
+constexpr int64_t kChainChildren = int64_t(1) << 21;
 constexpr int kMarchBlock = 256;
 constexpr int kMarchBlocksPerSm = 12;
 constexpr char kBadInput[] = "invalid field or source values (n_H < 0, x outside [0,1], non-finite, bad source)";
@@ -581,7 +581,7 @@ int grow_sources(rt_handle* h, int64_t need)
     e = e ? e : alloc((void**)&nw.ndot_a, 8 * (size_t)cap);
     e = e ? e : alloc((void**)&nw.cells_b, 12 * (size_t)cap);
     e = e ? e : alloc((void**)&nw.ndot_b, 8 * (size_t)cap);
-    e = e ? e : alloc((void**)&nw.label, 4 * (size_t)cap);
+    e = e ? e : alloc(&nw.pairs, pair_bytes(cap));
     e = e ? e : alloc((void**)&nw.parent, 4 * (size_t)cap);
     e = e ? e : alloc((void**)&nw.radius, 8 * (size_t)cap);
     e = e ? e : alloc((void**)&nw.count, 16);
@@ -589,7 +589,7 @@ int grow_sources(rt_handle* h, int64_t need)
     e = e ? e : alloc((void**)&emit, sizeof(SrcEntry) * (size_t)cap);
     auto release = [h](SourceWork& w) {
         void* ps[] = {w.cells_raw, w.ndot_raw, w.keys, w.keys_b, w.keys_c, w.order, w.order_b, w.flag, w.head_pos,
-                      w.cells_a, w.ndot_a, w.cells_b, w.ndot_b, w.label, w.parent, w.radius, w.count};
+                      w.cells_a, w.ndot_a, w.cells_b, w.ndot_b, w.pairs, w.parent, w.radius, w.count};
         for (void* q : ps) dfree(h, q);
     };
     if (e != cudaSuccess) {
@@ -646,7 +646,7 @@ int launch_level(rt_handle* h, int level, int64_t c0, int64_t c1, bool counted, 
     a.c1 = c1;
     a.in_count = counted && level > 0 ? h->d_count + level : nullptr;
     if (level == 0) {
-        a.src_count = h->n_emit < 0 ? h->sw.count : nullptr;
+        a.src_count = h->n_emit < 0 ? h->d_emit_count : nullptr;
         a.bad_input = &h->d_st->bad_input;
     }
     a.early = early;
@@ -790,64 +790,50 @@ int trace(rt_handle* h, const double* xuse, bool first)
     return RT_OK;
 }
 
-// Sec. 2.8 source stage of a step: validation of device-resident inputs,
-// dedup + sort, the n_th default, Alg. 3 merging when on, and the emitted
-// catalog (h->d_emit, h->n_emit). Leaves the field check in h->h_chk.
-int prepare_sources(rt_handle* h, bool wait, bool* merged_out, int64_t* n_dedup_out)
+// Sec. 2.8 source stage of a step: validation of the inputs, dedup + sort, Alg. 3 merging when on, and
+// the emitted catalog (h->d_emit). Everything is enqueued; the host learns the sizes in finish_sources.
+int prepare_sources(rt_handle* h)
 {
     NvtxRange nvtx("source stage (dedup, sort, Alg. 3)");
     cudaStream_t s = h->stream;
-    *merged_out = false;
-    h->catalog_valid = false;            // the buffers below are rewritten; valid again once emitted
-    // ---- validation of device-resident inputs
-    {
-        const int rc = enqueue_field_check(h);
-        if (rc) return rc;
+    h->catalog_valid = false;            // the buffers below are rewritten; valid again once a step has traced them
+    h->merged = false;
+    h->n_emit = h->n_dedup = 0;
+    int rc = enqueue_field_check(h);
+    if (rc) return rc;
+    bool merge = h->cfg.merge_mode == RT_MERGE_FORCED;
+    if (h->cfg.merge_mode == RT_MERGE_AUTO && h->nsrc > 0) {
+        RT_CUDA(h, cudaMemcpyAsync(h->h_chk, h->d_chk, sizeof(FieldCheck), cudaMemcpyDeviceToHost, s), "check read");
+        RT_CUDA(h, cudaStreamSynchronize(s), "source stage");
+        if (h->h_chk->bad) return fail(h, RT_EINVAL, kBadInput);
+        merge = h->h_chk->sum_x / (double)h->ncell > h->cfg.automerge_xbar;
     }
-    h->launches += launch_validate_sources(h->sw.cells_raw, h->sw.ndot_raw, h->nsrc, h->cfg.n, h->d_st, s);
-    RT_LAUNCHED(h, "validation launch");
-
-    // ---- sources: dedup + sort (Sec. 2.8)
-    h->launches += launch_dedup_sort(h->sw, h->nsrc, h->cfg.n, s);
+    if (h->nsrc <= 0) return RT_OK;
+    h->merged = merge;
+    h->launches += launch_sources(h->sw, h->nsrc, h->cfg.n, h->s_over_dx2, merge ? nullptr : h->d_emit, h->d_st, s);
     RT_LAUNCHED(h, "source launch");
-    if (!wait && h->cfg.merge_mode == RT_MERGE_OFF) {
-        h->launches += launch_build_emit_dev(h->sw, h->nsrc, h->s_over_dx2, h->d_emit, h->d_st, s);
-        RT_LAUNCHED(h, "emit launch");
-        h->n_emit = h->nsrc > 0 ? -1 : 0;
-        return RT_OK;
-    }
-    RT_CUDA(h, cudaMemcpyAsync(h->h_st, h->d_st, sizeof(DevStats), cudaMemcpyDeviceToHost, s), "stats read");
-    if (h->nsrc > 0)
-        RT_CUDA(h, cudaMemcpyAsync(h->h_i32, h->sw.count, sizeof(int32_t), cudaMemcpyDeviceToHost, s), "count read");
-    RT_CUDA(h, cudaMemcpyAsync(h->h_chk, h->d_chk, sizeof(FieldCheck), cudaMemcpyDeviceToHost, s), "check read");
-    RT_CUDA(h, cudaStreamSynchronize(s), "source stage");
-    if (h->h_st->bad_input || h->h_chk->bad) return fail(h, RT_EINVAL, kBadInput);
-    int64_t m = h->nsrc > 0 ? h->h_i32[0] : 0;
-    *n_dedup_out = m;
-    const double xbar = h->h_chk->sum_x / (double)h->ncell;
-
-    // ---- Alg. 3 source merging
-    if (m > 0 && (h->cfg.merge_mode == RT_MERGE_FORCED ||
-                  (h->cfg.merge_mode == RT_MERGE_AUTO && xbar > h->cfg.automerge_xbar))) {
+    if (merge) {
         const int Ls = h->cfg.merge_samp_level;
-        h->launches += launch_merge(h->sw, m, h->cfg.n, h->cfg.periodic, h->d_x, h->dirs + healpix_level_offset(Ls),
-                                    (int)(12 * (int64_t(1) << (2 * Ls))), h->cfg.merge_x_th, h->cfg.merge_f_req,
-                                    h->cfg.merge_n_min, h->cfg.merge_dr_cells, h->cfg.merge_rmax_cells,
-                                    h->cfg.merge_f_ov, h->cfg.merge_eps, h->d_st, s);
+        const MergeParams p{h->cfg.merge_x_th, h->cfg.merge_f_req, h->cfg.merge_n_min, h->cfg.merge_dr_cells,
+                            h->cfg.merge_rmax_cells, h->cfg.merge_f_ov, h->cfg.merge_eps};
+        h->launches += launch_merge(h->sw, h->nsrc, h->cfg.n, h->cfg.periodic, h->d_x,
+                                    h->dirs + healpix_level_offset(Ls), (int)(12 * (int64_t(1) << (2 * Ls))), p,
+                                    h->s_over_dx2, h->d_emit, h->d_st, s);
         RT_LAUNCHED(h, "merge launch");
-        RT_CUDA(h, cudaMemcpyAsync(h->h_i32, h->sw.count, sizeof(int32_t), cudaMemcpyDeviceToHost, s), "count read");
-        RT_CUDA(h, cudaMemcpyAsync(h->h_i32 + 1, &h->d_st->err, sizeof(unsigned), cudaMemcpyDeviceToHost, s), "err read");
-        RT_CUDA(h, cudaStreamSynchronize(s), "merge");
-        if (h->h_i32[1]) return fail(h, RT_EDEVICE, "source merge reported an internal error");
-        m = h->h_i32[0];
-        *merged_out = true;
     }
-    h->launches += launch_build_emit(h->sw, m, h->s_over_dx2, h->d_emit, h->d_st, s);
-    RT_LAUNCHED(h, "emit launch");
-    h->n_emit = m;
-    h->catalog_valid = true;
-
+    h->d_emit_count = merge ? h->sw.count + 2 : h->sw.count;
+    h->n_emit = -1;
     return RT_OK;
+}
+
+// The catalog's sizes, from sw.count as read back into h_i32 (the stream has been waited for).
+void finish_sources(rt_handle* h)
+{
+    if (h->n_emit < 0) {
+        h->n_dedup = h->h_i32[0];
+        h->n_emit = h->merged ? h->h_i32[2] : h->h_i32[0];
+    }
+    h->catalog_valid = true;
 }
 
 // Re-target an idle handle to a new configuration with the same grid size,
@@ -886,14 +872,15 @@ int sources_enqueue_many(rt_handle* const* hs, int count, int* rcs)
             const int rc = enqueue_field_check(h);
             if (rc) return rc;
         }
-        h->launches += launch_validate_sources(h->sw.cells_raw, h->sw.ndot_raw, h->nsrc, h->cfg.n, h->d_st, s);
-        h->launches += launch_dedup_sort(h->sw, h->nsrc, h->cfg.n, s);
-        if (h->nsrc > 0) h->launches += launch_build_emit_dev(h->sw, h->nsrc, h->s_over_dx2, h->d_emit, h->d_st, s);
+        h->launches += launch_sources(h->sw, h->nsrc, h->cfg.n, h->s_over_dx2, h->d_emit, h->d_st, s);
+        h->merged = false;
+        h->n_emit = h->nsrc > 0 ? -1 : 0;
+        h->n_dedup = 0;
         // statistics, count and mean written into the pinned block by a kernel (a server's result
         // copies of other requests may occupy the copy engines)
         ReadbackList rb;
         rb.add(h->d_st, pinned_dev(h, h->h_st), sizeof(DevStats));
-        if (h->nsrc > 0) rb.add(h->sw.count, pinned_dev(h, h->h_i32), sizeof(int32_t));
+        if (h->nsrc > 0) rb.add(h->sw.count, pinned_dev(h, h->h_i32), 4 * sizeof(int32_t));
         rb.add(h->d_chk, pinned_dev(h, h->h_chk), sizeof(FieldCheck));
         h->launches += launch_readback(rb, s);
         RT_LAUNCHED(h, "source stage launch");
@@ -921,12 +908,10 @@ int sources_wait_many(rt_handle* const* hs, int count, int* rcs)
         }
         if (rcs[i] != RT_OK) { ++failed; continue; }
         if (h->src_ready) continue;
-        const int64_t m = h->nsrc > 0 ? h->h_i32[0] : 0;
-        h->n_emit = m;
-        h->catalog_valid = true;
+        finish_sources(h);
         h->src_ready = true;
         h->src_merged = false;
-        h->src_dedup = m;
+        h->src_dedup = h->n_dedup;
         h->src_nth = h->cfg.n_th_cm3 >= 0 ? h->cfg.n_th_cm3 : h->h_chk->n_th;
         h->src_emitted = h->h_st->emitted;
     }
@@ -939,15 +924,19 @@ int handle_prepare_sources(rt_handle* h)
 {
     h->launches = 0;
     RT_CUDA(h, cudaMemsetAsync(h->d_st, 0, sizeof(DevStats), h->stream), "stats clear");
-    bool merged = false;
-    int64_t nd = 0;
-    const int rc = prepare_sources(h, true, &merged, &nd);
+    const int rc = prepare_sources(h);
     if (rc) return rc;
+    if (h->nsrc > 0)
+        RT_CUDA(h, cudaMemcpyAsync(h->h_i32, h->sw.count, 4 * sizeof(int32_t), cudaMemcpyDeviceToHost, h->stream), "counts");
+    RT_CUDA(h, cudaMemcpyAsync(h->h_chk, h->d_chk, sizeof(FieldCheck), cudaMemcpyDeviceToHost, h->stream), "check read");
     RT_CUDA(h, cudaMemcpyAsync(h->h_st, h->d_st, sizeof(DevStats), cudaMemcpyDeviceToHost, h->stream), "stats");
     RT_CUDA(h, cudaStreamSynchronize(h->stream), "source stage");
+    if (h->h_st->bad_input || h->h_chk->bad) return fail(h, RT_EINVAL, kBadInput);
+    if (h->h_st->err) return fail(h, RT_EDEVICE, "source merge reported an internal error");
+    finish_sources(h);
     h->src_ready = true;
-    h->src_merged = merged;
-    h->src_dedup = nd;
+    h->src_merged = h->merged;
+    h->src_dedup = h->n_dedup;
     h->src_nth = h->cfg.n_th_cm3 >= 0 ? h->cfg.n_th_cm3 : h->h_chk->n_th;
     h->src_emitted = h->h_st->emitted;
     return RT_OK;
@@ -1065,7 +1054,7 @@ int rt_destroy(rt_handle* h)
         for (void* q : ps) dfree(h, q);
         SourceWork& w = h->sw;
         void* ws[] = {w.cells_raw, w.ndot_raw, w.keys, w.keys_b, w.keys_c, w.order, w.order_b, w.flag, w.head_pos,
-                      w.cells_a, w.ndot_a, w.cells_b, w.ndot_b, w.label, w.parent, w.radius, w.count};
+                      w.cells_a, w.ndot_a, w.cells_b, w.ndot_b, w.pairs, w.parent, w.radius, w.count};
         for (void* q : ws) dfree(h, q);
         for (auto& r : h->rays) dfree(h, r.base);
     }
@@ -1363,7 +1352,6 @@ int rt_get_x(rt_handle* h, double* x_out, int where)
 static int reject(rt_handle* h)
 {
     h->n_emit = 0;
-    h->catalog_valid = false;
     return fail(h, RT_EINVAL, kBadInput);
 }
 
@@ -1382,10 +1370,8 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
     RT_CUDA(h, cudaMemsetAsync(h->d_st, 0, sizeof(DevStats), s), "stats clear");
     RT_CUDA(h, cudaEventRecord(h->ev[0], s), "event");
 
-    bool merged = false;
-    int64_t n_dedup = 0;
     {
-        const int rc = prepare_sources(h, false, &merged, &n_dedup);
+        const int rc = prepare_sources(h);
         if (rc) return rc;
     }
     h->ms_march = 0.0;
@@ -1461,22 +1447,20 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
     if (heat_out && !heat_direct) RT_CUDA(h, cudaMemcpyAsync(heat_out, h->d_heat, fb, k, s), "heat copy");
     RT_CUDA(h, cudaEventRecord(h->ev[3], s), "event");
     RT_CUDA(h, cudaMemcpyAsync(h->h_st, h->d_st, sizeof(DevStats), cudaMemcpyDeviceToHost, s), "stats read");
+    if (h->n_emit < 0)
+        RT_CUDA(h, cudaMemcpyAsync(h->h_i32, h->sw.count, 4 * sizeof(int32_t), cudaMemcpyDeviceToHost, s), "counts");
     RT_CUDA(h, cudaStreamSynchronize(s), "step");
     if (h->h_st->bad_input) return reject(h);
     if (h->h_st->err) return fail(h, RT_EDEVICE, "a kernel reported an internal error");
-    if (h->n_emit < 0) {                      // counted on the device, without merging
-        h->n_emit = h->h_st->n_emit;
-        n_dedup = h->n_emit;
-    }
-    h->catalog_valid = true;
+    finish_sources(h);
 
     if (st) {
         std::memset(st, 0, sizeof(*st));
         const DevStats& d = *h->h_st;
         st->n_src_in = h->nsrc;
-        st->n_src_dedup = n_dedup;
+        st->n_src_dedup = h->n_dedup;
         st->n_src_emit = h->n_emit;
-        st->merged = merged ? 1 : 0;
+        st->merged = h->merged ? 1 : 0;
         st->chem_iters = iters;
         st->level_max = h->level_max;
         st->launches = h->launches;

@@ -112,7 +112,10 @@ struct rt_handle {
     nyx::SourceWork sw;
     int64_t nsrc = 0;
     nyx::SrcEntry* d_emit = nullptr;
-    int64_t n_emit = 0;
+    int64_t n_emit = 0;                      // -1: still on the device
+    int64_t n_dedup = 0;
+    bool merged = false;
+    const int32_t* d_emit_count = nullptr;   // of sw.count
     bool catalog_valid = false;              // cells_a/ndot_a[0..n_emit) hold the catalog last traced
 
     nyx::RayStore rays[RT_MAX_LEVELS + 1];
@@ -152,9 +155,10 @@ inline T* pinned_dev(const rt_handle* h, T* host)
 {
     return reinterpret_cast<T*>(h->d_pin + (reinterpret_cast<char*>(host) - static_cast<char*>(h->h_pin)));
 }
-// The source stage of a step. Without merging it is only enqueued: the catalog's size then stays on the
-// device (h->n_emit is -1 until the step has ended) and invalid inputs show in DevStats::bad_input.
-int prepare_sources(rt_handle* h, bool wait, bool* merged_out, int64_t* n_dedup_out);
+// The source stage, enqueued: the catalog's size stays on the device (h->d_emit_count; h->n_emit is -1
+// until finish_sources), invalid inputs show in DevStats::bad_input and the field check. Waits only where
+// automatic merging has to know the mean of x.
+int prepare_sources(rt_handle* h);
 int ensure_directions(int device, int level, const int4** out, std::string& err);
 // The geometry table of a level for grids of n cells, with the entries of the FP32 march (fp64
 // false) or the FP64 one, built on stream s if needed; false if the level has none for that

@@ -46,8 +46,6 @@ struct DevStats {
     double maxdiff;                  // chemistry: max |<x>_new - <x>_old| (as ordered bits)
     unsigned int err;                // RT_ERR_* bits set by kernels
     unsigned int bad_input;          // count of invalid field / source values
-    int n_emit;                      // sources traced
-    int pad_;
 };
 
 // What one pass over a handle's fields finds.
@@ -248,27 +246,28 @@ struct SourceWork {
     double* ndot_a = nullptr;       // cap
     int32_t* cells_b = nullptr;     // cap x 3: merge scratch
     double* ndot_b = nullptr;       // cap
-    int32_t* label = nullptr;       // cap: union-find root of each source
+    void* pairs = nullptr;          // pair_bytes(cap): Alg. 3's shell tables, then the sources of its pair test
     int* parent = nullptr;          // cap: union-find forest
     double* radius = nullptr;       // cap: Alg. 3 bubble radii
     int32_t* count = nullptr;       // device scalars [4]
     int64_t cap = 0;
 };
-int launch_validate_sources(const int32_t* cells, const double* ndot, int64_t nsrc, int n, DevStats* st,
-                             cudaStream_t s);
-// Dedup + lexicographic sort (cells of an n^3 grid); writes cells_a/ndot_a and count[0] = number
-// of unique cells.
-int launch_dedup_sort(SourceWork& w, int64_t nsrc, int n, cudaStream_t s);
-// Alg. 3 on cells_a/ndot_a[0..m): radii, union-find, merged catalog into cells_a/ndot_a, count[0] = size.
-int launch_merge(SourceWork& w, int64_t m, int n, int periodic, const double* x, const int4* samp_dirs,
-                 int samp_count, double x_th, double f_req, int n_min, double dr, double rmax, double f_ov,
-                 double eps, DevStats* st, cudaStream_t s);
-// Emitted catalog entries from cells_a/ndot_a[0..*count) with *count read on the device (<= max_m).
-int launch_build_emit_dev(const SourceWork& w, int64_t max_m, double s_over_dx2, SrcEntry* out, DevStats* st,
-                          cudaStream_t s);
-// Emitted catalog entries from cells_a/ndot_a[0..m).
-int launch_build_emit(const SourceWork& w, int64_t m, double s_over_dx2, SrcEntry* out, DevStats* st,
-                      cudaStream_t s);
+inline size_t pair_bytes(int64_t cap) { return (size_t)(cap > 16384 ? 16 * cap : 16 * 16384); }
+// Validation (into st->bad_input), dedup and lexicographic sort (cells of an n^3 grid): cells_a/ndot_a,
+// their number in count[0], and the emitted entries (emit null: none).
+int launch_sources(SourceWork& w, int64_t nsrc, int n, double s_over_dx2, SrcEntry* emit, DevStats* st, cudaStream_t s);
+// Emitted entries of cells_a/ndot_a[0..*count) (<= bound).
+int launch_emit(const SourceWork& w, int64_t bound, const int32_t* count, double s_over_dx2, SrcEntry* emit,
+                DevStats* st, cudaStream_t s);
+// Alg. 3 on cells_a/ndot_a[0..count[0]) (<= bound): radii, union-find, merged catalog into
+// cells_a/ndot_a and emit, its size in count[2].
+struct MergeParams {
+    double x_th, f_req;
+    int n_min;
+    double dr, rmax, f_ov, eps;
+};
+int launch_merge(SourceWork& w, int64_t bound, int n, int periodic, const double* x, const int4* samp_dirs,
+                 int samp_count, const MergeParams& p, double s_over_dx2, SrcEntry* emit, DevStats* st, cudaStream_t s);
 
 // directions.cpp: quantised HEALPix nested pixel centres, levels 0..max_level
 // concatenated (offset of level l = 12 (4^l - 1) / 3). Host memory.

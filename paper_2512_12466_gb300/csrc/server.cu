@@ -64,7 +64,7 @@ struct SrvReq {
 int64_t handle_bytes(int n, int precision, int64_t src_cap)
 {
     const int64_t cells = (int64_t)n * n * n;
-    return cells * (32 + (precision == RT_FP32 ? 4 : 8)) + 160 * std::max<int64_t>(src_cap, 1024) + (1 << 16);
+    return cells * (32 + (precision == RT_FP32 ? 4 : 8)) + 172 * std::max<int64_t>(src_cap, 1024) + (3 << 17);
 }
 
 // Source capacity a handle with capacity cap has after taking nsrc sources
