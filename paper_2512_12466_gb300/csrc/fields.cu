@@ -99,16 +99,22 @@ __global__ void __launch_bounds__(kBlock) check_fields_kernel(const double* __re
         }
     }
     bad = __reduce_add_sync(0xffffffffu, bad);
-    if ((threadIdx.x & 31) == 0 && bad) atomicAdd(&chk->bad, bad);
-    sn = block_sum(sn);
+    if ((threadIdx.x & 31) == 0 && bad) atomicAdd(&chk->acc_bad, bad);
+    sn = block_sum(sn);                       // its barriers also order the counts of bad cells
     if (want_x) sx = block_sum(sx);
     if (threadIdx.x == 0) {
-        atomicAdd(&chk->sum_nh, sn);
-        if (want_x) atomicAdd(&chk->sum_x, sx);
+        atomicAdd(&chk->acc_nh, sn);
+        if (want_x) atomicAdd(&chk->acc_x, sx);
         __threadfence();
         if (atomicAdd(&chk->blocks_done, 1u) + 1u == gridDim.x) {
-            const double total = *((volatile double*)&chk->sum_nh);
+            __threadfence();
+            const double total = *((volatile double*)&chk->acc_nh);
+            chk->sum_nh = total;
+            chk->sum_x = *((volatile double*)&chk->acc_x);
             chk->n_th = __dmul_rn(0.01, __ddiv_rn(total, (double)ncell));
+            chk->bad = *((volatile unsigned*)&chk->acc_bad);
+            chk->acc_nh = chk->acc_x = 0.0;
+            chk->acc_bad = chk->blocks_done = 0u;
         }
     }
 }

@@ -584,12 +584,12 @@ int grow_sources(rt_handle* h, int64_t need)
     e = e ? e : alloc(&nw.pairs, pair_bytes(cap));
     e = e ? e : alloc((void**)&nw.parent, 4 * (size_t)cap);
     e = e ? e : alloc((void**)&nw.radius, 8 * (size_t)cap);
-    e = e ? e : alloc((void**)&nw.count, 16);
+    nw.count = h->d_words->src_count;
     SrcEntry* emit = nullptr;
     e = e ? e : alloc((void**)&emit, sizeof(SrcEntry) * (size_t)cap);
     auto release = [h](SourceWork& w) {
         void* ps[] = {w.cells_raw, w.ndot_raw, w.keys, w.keys_b, w.keys_c, w.order, w.order_b, w.flag, w.head_pos,
-                      w.cells_a, w.ndot_a, w.cells_b, w.ndot_b, w.pairs, w.parent, w.radius, w.count};
+                      w.cells_a, w.ndot_a, w.cells_b, w.ndot_b, w.pairs, w.parent, w.radius};
         for (void* q : ps) dfree(h, q);
     };
     if (e != cudaSuccess) {
@@ -701,8 +701,9 @@ int run_levels(rt_handle* h, int level, int64_t total, bool counted)
         return fail(h, RT_EDEVICE, "ray level beyond the direction table");
     for (int64_t c0 = 0; c0 < total; c0 += kMaxChildrenPerLaunch) {
         const int64_t c1 = std::min(total, c0 + kMaxChildrenPerLaunch);
-        RT_CUDA(h, cudaMemsetAsync(h->d_count + level + 1, 0, sizeof(unsigned long long) * (size_t)(RT_MAX_LEVELS - level),
-                                   h->stream), "counters");
+        if (level > 0 || c0 > 0)             // the step's first launch finds them cleared
+            RT_CUDA(h, cudaMemsetAsync(h->d_count + level + 1, 0,
+                                       sizeof(unsigned long long) * (size_t)(RT_MAX_LEVELS - level), h->stream), "counters");
         int l = level;
         int64_t bound = c1 - c0;
         int rc = launch_level<R>(h, l, c0, c1, counted, false);
@@ -714,13 +715,11 @@ int run_levels(rt_handle* h, int level, int64_t total, bool counted)
             if (rc) return rc;
         }
         if (l == h->table_level) continue;
-        RT_CUDA(h, cudaMemcpyAsync(h->h_count + l + 1, h->d_count + l + 1, sizeof(unsigned long long),
-                                   cudaMemcpyDeviceToHost, h->stream), "counter read");
-        RT_CUDA(h, cudaMemcpyAsync(h->h_i32, &h->d_st->err, sizeof(unsigned), cudaMemcpyDeviceToHost, h->stream),
-                "error read");
+        RT_CUDA(h, cudaMemcpyAsync(h->h_words, h->d_words, sizeof(StepWords), cudaMemcpyDeviceToHost, h->stream), "counter read");
         RT_CUDA(h, cudaStreamSynchronize(h->stream), "march");
-        if (h->h_i32[0]) return fail(h, RT_EDEVICE, "march kernel reported an internal error");
-        rc = run_levels<R>(h, l + 1, 4 * (int64_t)h->h_count[l + 1], false);
+        if (h->h_st->bad_input) return RT_OK;                  // nothing was traced; the step ends with the error
+        if (h->h_st->err) return fail(h, RT_EDEVICE, "march kernel reported an internal error");
+        rc = run_levels<R>(h, l + 1, 4 * (int64_t)h->h_words->ray_count[l + 1], false);
         if (rc) return rc;
     }
     return RT_OK;
@@ -747,7 +746,6 @@ int enqueue_field_check(rt_handle* h)
 {
     const bool want_x = h->cfg.merge_mode == RT_MERGE_AUTO;
     if (h->fields_checked && (h->checked_x || !want_x)) return RT_OK;
-    RT_CUDA(h, cudaMemsetAsync(h->d_chk, 0, sizeof(FieldCheck), h->stream), "check clear");
     h->launches += launch_check_fields(h->d_nh, h->d_x, h->ncell, nullptr, nullptr, want_x, h->d_chk, h->stream);
     RT_LAUNCHED(h, "check launch");
     h->fields_checked = true;
@@ -771,8 +769,11 @@ bool direct_access(const rt_handle* h, const void* p)
 // first: the step's first trace, with the statistics as rt_step cleared them.
 int trace(rt_handle* h, const double* xuse, bool first)
 {
-    // per-trace part of the statistics: per-level counters, hash and ledger
-    if (!first) RT_CUDA(h, cudaMemsetAsync(h->d_st, 0, offsetof(DevStats, deposited), h->stream), "stats clear");
+    // counters of the levels and the per-trace part of the statistics: per-level counters, hash and ledger
+    if (!first)
+        RT_CUDA(h, cudaMemsetAsync(h->d_words->ray_count, 0,
+                                   offsetof(StepWords, st) + offsetof(DevStats, deposited) - offsetof(StepWords, ray_count),
+                                   h->stream), "stats clear");
     FieldJob job = field_job(h, xuse);
     job.valid = first ? h->d_chk : nullptr;
     launch_prepare_kappa(job, h->cfg.precision == RT_FP32, h->stream);
@@ -826,12 +827,12 @@ int prepare_sources(rt_handle* h)
     return RT_OK;
 }
 
-// The catalog's sizes, from sw.count as read back into h_i32 (the stream has been waited for).
+// The catalog's sizes, from h_words as read back (the stream has been waited for).
 void finish_sources(rt_handle* h)
 {
     if (h->n_emit < 0) {
-        h->n_dedup = h->h_i32[0];
-        h->n_emit = h->merged ? h->h_i32[2] : h->h_i32[0];
+        h->n_dedup = h->h_words->src_count[0];
+        h->n_emit = h->h_words->src_count[h->merged ? 2 : 0];
     }
     h->catalog_valid = true;
 }
@@ -879,8 +880,7 @@ int sources_enqueue_many(rt_handle* const* hs, int count, int* rcs)
         // statistics, count and mean written into the pinned block by a kernel (a server's result
         // copies of other requests may occupy the copy engines)
         ReadbackList rb;
-        rb.add(h->d_st, pinned_dev(h, h->h_st), sizeof(DevStats));
-        if (h->nsrc > 0) rb.add(h->sw.count, pinned_dev(h, h->h_i32), 4 * sizeof(int32_t));
+        rb.add(h->d_words, pinned_dev(h, h->h_words), sizeof(StepWords));
         rb.add(h->d_chk, pinned_dev(h, h->h_chk), sizeof(FieldCheck));
         h->launches += launch_readback(rb, s);
         RT_LAUNCHED(h, "source stage launch");
@@ -926,10 +926,8 @@ int handle_prepare_sources(rt_handle* h)
     RT_CUDA(h, cudaMemsetAsync(h->d_st, 0, sizeof(DevStats), h->stream), "stats clear");
     const int rc = prepare_sources(h);
     if (rc) return rc;
-    if (h->nsrc > 0)
-        RT_CUDA(h, cudaMemcpyAsync(h->h_i32, h->sw.count, 4 * sizeof(int32_t), cudaMemcpyDeviceToHost, h->stream), "counts");
     RT_CUDA(h, cudaMemcpyAsync(h->h_chk, h->d_chk, sizeof(FieldCheck), cudaMemcpyDeviceToHost, h->stream), "check read");
-    RT_CUDA(h, cudaMemcpyAsync(h->h_st, h->d_st, sizeof(DevStats), cudaMemcpyDeviceToHost, h->stream), "stats");
+    RT_CUDA(h, cudaMemcpyAsync(h->h_words, h->d_words, sizeof(StepWords), cudaMemcpyDeviceToHost, h->stream), "stats");
     RT_CUDA(h, cudaStreamSynchronize(h->stream), "source stage");
     if (h->h_st->bad_input || h->h_chk->bad) return fail(h, RT_EINVAL, kBadInput);
     if (h->h_st->err) return fail(h, RT_EDEVICE, "source merge reported an internal error");
@@ -1050,11 +1048,11 @@ int rt_destroy(rt_handle* h)
     cudaStreamSynchronize(h->stream);
     {
         void* ps[] = {h->d_nh, h->d_x, h->d_xavg, h->d_xend, h->d_gamma, h->d_heat, h->d_kap, h->d_chk,
-                      h->d_emit, h->d_count, h->d_st};
+                      h->d_emit, h->d_words};
         for (void* q : ps) dfree(h, q);
         SourceWork& w = h->sw;
         void* ws[] = {w.cells_raw, w.ndot_raw, w.keys, w.keys_b, w.keys_c, w.order, w.order_b, w.flag, w.head_pos,
-                      w.cells_a, w.ndot_a, w.cells_b, w.ndot_b, w.pairs, w.parent, w.radius, w.count};
+                      w.cells_a, w.ndot_a, w.cells_b, w.ndot_b, w.pairs, w.parent, w.radius};
         for (void* q : ws) dfree(h, q);
         for (auto& r : h->rays) dfree(h, r.base);
     }
@@ -1092,20 +1090,21 @@ int rt_create(const rt_config* cfg, void* cuda_stream, rt_handle** out)
         e = e ? e : dalloc(h, (void**)&h->d_xend, fb);
     }
     e = e ? e : dalloc(h, (void**)&h->d_chk, sizeof(FieldCheck));
-    e = e ? e : dalloc(h, (void**)&h->d_count, sizeof(unsigned long long) * (RT_MAX_LEVELS + 1));
-    e = e ? e : dalloc(h, (void**)&h->d_st, sizeof(DevStats));
+    e = e ? e : dalloc(h, (void**)&h->d_words, sizeof(StepWords));
+    e = e ? e : cudaMemsetAsync(h->d_chk, 0, sizeof(FieldCheck), h->stream);
+    if (e == cudaSuccess) {
+        h->d_count = h->d_words->ray_count;
+        h->d_st = &h->d_words->st;
+    }
     {   // one pinned block for every host-side readback
-        const size_t a = (sizeof(DevStats) + 63) & ~size_t(63);
-        const size_t b = (sizeof(unsigned long long) * (RT_MAX_LEVELS + 1) + 63) & ~size_t(63);
-        e = e ? e : cudaMallocHost(&h->h_pin, a + b + 192);
+        const size_t a = (sizeof(StepWords) + 63) & ~size_t(63);
+        e = e ? e : cudaMallocHost(&h->h_pin, a + sizeof(FieldCheck));
         e = e ? e : cudaHostGetDevicePointer(reinterpret_cast<void**>(&h->d_pin), h->h_pin, 0);
         if (e == cudaSuccess) {
             char* q = static_cast<char*>(h->h_pin);
-            h->h_st = reinterpret_cast<DevStats*>(q);
-            h->h_count = reinterpret_cast<unsigned long long*>(q + a);
-            h->h_i32 = reinterpret_cast<int32_t*>(q + a + b);
-            h->h_f64 = reinterpret_cast<double*>(q + a + b + 64);
-            h->h_chk = reinterpret_cast<FieldCheck*>(q + a + b + 128);
+            h->h_words = reinterpret_cast<StepWords*>(q);
+            h->h_st = &h->h_words->st;
+            h->h_chk = reinterpret_cast<FieldCheck*>(q + a);
         }
     }
     for (auto& ev : h->ev) e = e ? e : cudaEventCreate(&ev);
@@ -1130,7 +1129,6 @@ int rt_set_fields(rt_handle* h, const double* n_H, const double* x_ion, int wher
     if (where == RT_DEVICE && direct_access(h, n_H) && direct_access(h, x_ion)) {
         // copied and checked in one pass
         const bool want_x = h->cfg.merge_mode == RT_MERGE_AUTO;
-        RT_CUDA(h, cudaMemsetAsync(h->d_chk, 0, sizeof(FieldCheck), h->stream), "check clear");
         launch_check_fields(n_H, x_ion, h->ncell, h->d_nh, h->d_x, want_x, h->d_chk, h->stream);
         RT_LAUNCHED(h, "field copy");
         h->fields_checked = true;
@@ -1165,6 +1163,12 @@ int rt_add_sources(rt_handle* h, const int32_t* cell_ijk, const double* ndot, in
     h->catalog_valid = false;
     int rc = grow_sources(h, h->nsrc + n);
     if (rc) return rc;
+    if (where == RT_DEVICE && direct_access(h, ndot) && direct_access(h, cell_ijk)) {
+        launch_copy_sources(cell_ijk, ndot, n, h->sw.cells_raw + 3 * h->nsrc, h->sw.ndot_raw + h->nsrc, h->stream);
+        RT_LAUNCHED(h, "source copy");
+        h->nsrc += n;
+        return RT_OK;
+    }
     const cudaMemcpyKind k = where == RT_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
     RT_CUDA(h, cudaMemcpyAsync(h->sw.cells_raw + 3 * h->nsrc, cell_ijk, 12 * (size_t)n, k, h->stream), "source copy");
     RT_CUDA(h, cudaMemcpyAsync(h->sw.ndot_raw + h->nsrc, ndot, 8 * (size_t)n, k, h->stream), "source copy");
@@ -1367,7 +1371,7 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
     cudaStream_t s = h->stream;
     h->launches = 0;
     h->err.clear();
-    RT_CUDA(h, cudaMemsetAsync(h->d_st, 0, sizeof(DevStats), s), "stats clear");
+    RT_CUDA(h, cudaMemsetAsync(h->d_words, 0, sizeof(StepWords), s), "stats clear");
     RT_CUDA(h, cudaEventRecord(h->ev[0], s), "event");
 
     {
@@ -1389,20 +1393,15 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
             int rc = trace(h, xuse, iters == 0);
             if (rc) return rc;
             ++iters;
-            RT_CUDA(h, cudaMemsetAsync(&h->d_st->maxdiff, 0, sizeof(double), s), "clear");
             h->launches += launch_chem_update(h->d_nh, h->d_x, xuse, xnew, h->d_xend, h->d_gamma, h->ncell, dt_s,
                                               h->cfg.alpha_B, h->cfg.C_H, h->cfg.clumping, h->d_st, s);
             RT_LAUNCHED(h, "chemistry launch");
-            // the residual, and the error words beside it
-            static_assert(offsetof(DevStats, bad_input) == offsetof(DevStats, maxdiff) + 12, "read together");
-            RT_CUDA(h, cudaMemcpyAsync(h->h_f64 + 2, &h->d_st->maxdiff, 2 * sizeof(double), cudaMemcpyDeviceToHost, s),
-                    "residual read");
+            // the residual, and the error words
+            RT_CUDA(h, cudaMemcpyAsync(h->h_words, h->d_words, sizeof(StepWords), cudaMemcpyDeviceToHost, s), "residual read");
             RT_CUDA(h, cudaStreamSynchronize(s), "chemistry");
-            resid = h->h_f64[2];
-            unsigned words[2];
-            std::memcpy(words, h->h_f64 + 3, sizeof(words));
-            if (words[1]) return reject(h);
-            if (words[0]) return fail(h, RT_EDEVICE, "march kernel reported an internal error");
+            resid = h->h_st->maxdiff;
+            if (h->h_st->bad_input) return reject(h);
+            if (h->h_st->err) return fail(h, RT_EDEVICE, "march kernel reported an internal error");
             float ms = 0.f;
             RT_CUDA(h, cudaEventElapsedTime(&ms, h->ev[1], h->ev[2]), "event");
             h->ms_march = ms;
@@ -1439,16 +1438,14 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
     const cudaMemcpyKind k = where == RT_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
     if ((gamma_out && !gamma_direct) || (heat_out && !heat_direct)) {
         // nothing is copied over the caller's data before the inputs are known to be valid
-        RT_CUDA(h, cudaMemcpyAsync(h->h_i32, &h->d_st->bad_input, sizeof(unsigned), cudaMemcpyDeviceToHost, s), "input check");
+        RT_CUDA(h, cudaMemcpyAsync(h->h_words, h->d_words, sizeof(StepWords), cudaMemcpyDeviceToHost, s), "input check");
         RT_CUDA(h, cudaStreamSynchronize(s), "step");
-        if (h->h_i32[0]) return reject(h);
+        if (h->h_st->bad_input) return reject(h);
     }
     if (gamma_out && !gamma_direct) RT_CUDA(h, cudaMemcpyAsync(gamma_out, h->d_gamma, fb, k, s), "gamma copy");
     if (heat_out && !heat_direct) RT_CUDA(h, cudaMemcpyAsync(heat_out, h->d_heat, fb, k, s), "heat copy");
     RT_CUDA(h, cudaEventRecord(h->ev[3], s), "event");
-    RT_CUDA(h, cudaMemcpyAsync(h->h_st, h->d_st, sizeof(DevStats), cudaMemcpyDeviceToHost, s), "stats read");
-    if (h->n_emit < 0)
-        RT_CUDA(h, cudaMemcpyAsync(h->h_i32, h->sw.count, 4 * sizeof(int32_t), cudaMemcpyDeviceToHost, s), "counts");
+    RT_CUDA(h, cudaMemcpyAsync(h->h_words, h->d_words, sizeof(StepWords), cudaMemcpyDeviceToHost, s), "stats read");
     RT_CUDA(h, cudaStreamSynchronize(s), "step");
     if (h->h_st->bad_input) return reject(h);
     if (h->h_st->err) return fail(h, RT_EDEVICE, "a kernel reported an internal error");

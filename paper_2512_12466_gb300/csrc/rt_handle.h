@@ -119,17 +119,16 @@ struct rt_handle {
     bool catalog_valid = false;              // cells_a/ndot_a[0..n_emit) hold the catalog last traced
 
     nyx::RayStore rays[RT_MAX_LEVELS + 1];
-    unsigned long long* d_count = nullptr;   // one per level
-    nyx::DevStats* d_st = nullptr;
-    void* h_pin = nullptr;                   // one pinned block holding the four below
+    nyx::StepWords* d_words = nullptr;
+    unsigned long long* d_count = nullptr;   // d_words->ray_count
+    nyx::DevStats* d_st = nullptr;           // &d_words->st
+    void* h_pin = nullptr;                   // one pinned block holding the two below
     char* d_pin = nullptr;                   // the same block's device address (mapped)
-    nyx::DevStats* h_st = nullptr;
-    unsigned long long* h_count = nullptr;
-    int32_t* h_i32 = nullptr;                // scratch
-    double* h_f64 = nullptr;                 // scratch
+    nyx::StepWords* h_words = nullptr;
+    nyx::DevStats* h_st = nullptr;           // &h_words->st
     nyx::FieldCheck* h_chk = nullptr;
 
-    cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
+    cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
     double ms_march = 0.0;
     bool fields_set = false;
     bool sticky = false;

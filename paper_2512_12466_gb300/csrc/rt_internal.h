@@ -40,10 +40,10 @@ struct DevStats {
     unsigned long long secondary[RT_MAX_LEVELS];
     unsigned long long visit_hash;
     double absorbed, escaped_ph, dropped_ph;
+    double maxdiff;                  // chemistry: max |<x>_new - <x>_old| (as ordered bits)
     // -- fields below survive the per-trace reset (which clears up to `deposited`)
     double deposited;
     double emitted;
-    double maxdiff;                  // chemistry: max |<x>_new - <x>_old| (as ordered bits)
     unsigned int err;                // RT_ERR_* bits set by kernels
     unsigned int bad_input;          // count of invalid field / source values
 };
@@ -53,7 +53,18 @@ struct FieldCheck {
     double sum_nh, sum_x;
     double n_th;                     // default threshold of Eqs. 7-8: 0.01 mean(n_H)
     unsigned bad;                    // cells with n_H < 0, x outside [0, 1] or a value that is not finite
+    // the pass's accumulators: zero before it, and again when its last block has published the above
+    unsigned acc_bad;
+    double acc_nh, acc_x;
     unsigned blocks_done;
+    unsigned pad_;
+};
+
+// A handle's small device words, one block that one clear and one read cover.
+struct StepWords {
+    int32_t src_count[4];                              // SourceWork::count
+    unsigned long long ray_count[RT_MAX_LEVELS + 1];   // parents of each level
+    DevStats st;
 };
 
 // The per-cell passes before and after a trace, for one solve.
@@ -195,7 +206,7 @@ void launch_geom_fill64(long long rq, int l, const int4* dirs, long long npix, i
                         unsigned* err, cudaStream_t s);
 
 // fields.cu
-// New fields: invalid values counted, n_H (and x, if want_x) summed into *chk (zeroed by the caller), and
+// New fields: invalid values counted, n_H (and x, if want_x) summed into *chk (its accumulators zero), and
 // copied where nh_out and x_out are given.
 int launch_check_fields(const double* nh, const double* x, int64_t ncell, double* nh_out, double* x_out, bool want_x,
                         FieldCheck* chk, cudaStream_t s);
@@ -256,6 +267,9 @@ inline size_t pair_bytes(int64_t cap) { return (size_t)(cap > 16384 ? 16 * cap :
 // Validation (into st->bad_input), dedup and lexicographic sort (cells of an n^3 grid): cells_a/ndot_a,
 // their number in count[0], and the emitted entries (emit null: none).
 int launch_sources(SourceWork& w, int64_t nsrc, int n, double s_over_dx2, SrcEntry* emit, DevStats* st, cudaStream_t s);
+// n sources appended: both arrays in one launch.
+int launch_copy_sources(const int32_t* cells, const double* ndot, int64_t n, int32_t* to_cells, double* to_ndot,
+                        cudaStream_t s);
 // Emitted entries of cells_a/ndot_a[0..*count) (<= bound).
 int launch_emit(const SourceWork& w, int64_t bound, const int32_t* count, double s_over_dx2, SrcEntry* emit,
                 DevStats* st, cudaStream_t s);
