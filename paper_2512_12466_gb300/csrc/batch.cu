@@ -22,7 +22,9 @@
 
 #include <algorithm>
 #include <cstring>
+#include <new>
 #include <string>
+#include <utility>
 #include <vector>
 
 #include "rt_handle.h"
@@ -49,6 +51,9 @@ constexpr int64_t kLaneRecordBytes = int64_t(768) << 20;
 // A solve that traced at least this many segments in its last run gets a launch of its own (the
 // single-solve kernel); lighter solves share launches, where batching pays.
 constexpr unsigned long long kHeavySegments = 1ULL << 26;
+// Segments that a launch of light solves may hold without regard to the L2-sized groups (4 M segments are
+// some 50 us of march).
+constexpr unsigned long long kLightSegments = 1ULL << 22;
 
 }  // namespace
 
@@ -83,6 +88,8 @@ struct rt_batch {
     std::vector<FieldJob> jobs;             // the solves' per-cell passes, then an end mark
     FieldJob* d_jobs = nullptr;
     uint32_t field_blocks = 0;
+    FieldOut* d_outs = nullptr;            // where the run's results go, from h_outs before every launch
+    FieldOut* h_outs = nullptr;            // pinned
     DevStats* d_stats = nullptr;
     DevStats* h_stats = nullptr;           // pinned
     DevStats* m_stats = nullptr;           // its device address (mapped)
@@ -338,7 +345,9 @@ int enqueue(rt_batch* b)
     B_CUDA(b, cudaGetLastError(), "kappa launch");
     B_CUDA(b, cudaMemsetAsync(b->d_stats, 0, sizeof(DevStats) * b->hs.size(), s), "stats clear");
     B_CUDA(b, cudaMemsetAsync(b->d_err, 0, sizeof(unsigned), s), "error clear");
-    // consecutive groups of solves whose kappa + Gamma fit the budget, one launch each; a solve
+    // consecutive groups of solves whose kappa + Gamma fit the budget, one launch each (solves that traced
+    // little in the last run, kLightSegments a launch in all, share one whatever their bytes: they touch few
+    // of their cells, and a launch costs 35 us); a solve
     // that fills half the budget or more, or traced many segments in the last run, runs alone (the
     // single-solve kernel, whose solve parameters are kernel parameters rather than per-lane loads)
     const int rbytes = b->precision == RT_FP32 ? 12 : 16;
@@ -361,6 +370,8 @@ int enqueue(rt_batch* b)
         }
         size_t i1 = i0;
         int64_t bytes = 0, srcs = 0;
+        unsigned long long segs = 0;
+        auto light = [&](size_t i) { return i < b->work.size() && b->work[i] > 0 && segs + b->work[i] <= kLightSegments; };
         // one rate per launch: gray, or the blackbody at one temperature
         auto same_rate = [&](size_t i) {
             const rt_config& a = b->hs[i0]->cfg;
@@ -369,8 +380,9 @@ int enqueue(rt_batch* b)
         };
         while (i1 < b->hs.size() && !hv[i1]) {
             const int64_t add = rbytes * b->hs[i1]->ncell;
-            if (i1 > i0 && (big(i0) || big(i1) || (gb > 0 && bytes + add > gb) || !same_rate(i1))) break;
+            if (i1 > i0 && (!same_rate(i1) || (!light(i1) && (big(i0) || big(i1) || (gb > 0 && bytes + add > gb))))) break;
             bytes += add;
+            segs += i1 < b->work.size() ? b->work[i1] : 0;
             srcs += b->n_emit[i1];
             ++i1;
         }
@@ -392,7 +404,7 @@ int enqueue(rt_batch* b)
         const int rc = enqueue_heavy(b, hv);
         if (rc) return rc;
     }
-    b->launches += launch_finalize_many(b->d_jobs, (int)b->hs.size(), b->field_blocks, s);
+    b->launches += launch_finalize_many(b->d_jobs, b->d_outs, (int)b->hs.size(), b->field_blocks, s);
     B_CUDA(b, cudaGetLastError(), "finalize launch");
     // statistics and error word written into pinned memory by a kernel, not copied: a server's
     // result copies of the previous batch may occupy the copy engines
@@ -450,6 +462,8 @@ int run_launch(rt_batch* b)
         const int rc = ensure_lanes(b);
         if (rc) return rc;
     }
+    B_CUDA(b, cudaMemcpyAsync(b->d_outs, b->h_outs, sizeof(FieldOut) * b->hs.size(), cudaMemcpyHostToDevice, b->stream),
+           "outputs");
     B_CUDA(b, cudaEventRecord(b->ev0, b->stream), "event");
     if (b->captured) {
         B_CUDA(b, cudaGraphLaunch(b->exec, b->stream), "graph launch");
@@ -662,7 +676,11 @@ int nyx::batch_bind(rt_batch* b, rt_handle* const* handles, int32_t count)
         if (b->d_stats) B_CUDA(b, cudaFreeAsync(b->d_stats, b->stream), "stats");
         if (b->d_solves) B_CUDA(b, cudaFreeAsync(b->d_solves, b->stream), "solve table");
         if (b->d_jobs) B_CUDA(b, cudaFreeAsync(b->d_jobs, b->stream), "field jobs");
+        if (b->d_outs) B_CUDA(b, cudaFreeAsync(b->d_outs, b->stream), "outputs");
+        cudaFreeHost(b->h_outs);
         b->d_jobs = nullptr;
+        b->d_outs = nullptr;
+        b->h_outs = nullptr;
         cudaFreeHost(b->h_stats);
         b->d_stats = nullptr;
         b->h_stats = nullptr;
@@ -674,6 +692,8 @@ int nyx::batch_bind(rt_batch* b, rt_handle* const* handles, int32_t count)
         B_CUDA(b, cudaHostGetDevicePointer(reinterpret_cast<void**>(&b->m_stats), b->h_stats, 0), "stats");
         B_CUDA(b, cudaMallocAsync(&b->d_solves, sizeof(BatchSolve) * (size_t)b->cap_solves, b->stream), "solve table");
         B_CUDA(b, cudaMallocAsync(&b->d_jobs, sizeof(FieldJob) * (size_t)(b->cap_solves + 1), b->stream), "field jobs");
+        B_CUDA(b, cudaMallocAsync(&b->d_outs, sizeof(FieldOut) * (size_t)b->cap_solves, b->stream), "outputs");
+        B_CUDA(b, cudaMallocHost(&b->h_outs, sizeof(FieldOut) * (size_t)b->cap_solves), "outputs");
     }
     b->hsolve.assign(b->hs.size(), BatchSolve{});
     b->jobs.clear();
@@ -682,7 +702,7 @@ int nyx::batch_bind(rt_batch* b, rt_handle* const* handles, int32_t count)
         FieldJob j = field_job(b->hs[i], b->hs[i]->d_x);
         j.n_th = b->n_th[i];
         j.chk = nullptr;
-        j.heat = b->hs[i]->d_heat;
+        b->h_outs[i] = {nullptr, b->hs[i]->d_heat};
         j.st = b->d_stats + i;
         j.block0 = b->field_blocks;
         b->field_blocks += field_blocks(j.ncell);
@@ -745,6 +765,7 @@ int rt_batch_destroy(rt_batch* b)
     if (b->stream) {
         if (b->d_solves) cudaFreeAsync(b->d_solves, b->stream);
         if (b->d_jobs) cudaFreeAsync(b->d_jobs, b->stream);
+        if (b->d_outs) cudaFreeAsync(b->d_outs, b->stream);
         if (b->d_stats) cudaFreeAsync(b->d_stats, b->stream);
         if (b->d_src) cudaFreeAsync(b->d_src, b->stream);
         cudaStreamSynchronize(b->stream);
@@ -752,6 +773,7 @@ int rt_batch_destroy(rt_batch* b)
     cudaFree(b->d_counts);
     cudaFree(b->d_tiles);
     cudaFree(b->d_err);
+    cudaFreeHost(b->h_outs);
     cudaFreeHost(b->h_stats);
     cudaFreeHost(b->h_err);
     if (b->ev0) cudaEventDestroy(b->ev0);
@@ -874,15 +896,44 @@ int rt_batch_run(rt_batch* b, double* const* gamma_out, double* const* heat_out,
     if (b->sticky) return RT_ESTATE;
     if (where != RT_HOST && where != RT_DEVICE) return bfail(b, RT_EINVAL, "bad where");
     DeviceGuard g(b->device);
+    // results go straight into the caller's device buffers, where a kernel may write them and no two
+    // overlap; the others are copied after the run
+    std::vector<std::pair<const double*, const double*>> spans;
+    std::vector<FieldOut> outs;
+    try {
+        outs.resize(b->hs.size());
+        for (size_t i = 0; where == RT_DEVICE && i < b->hs.size(); ++i) {
+            if (gamma_out && gamma_out[i]) spans.emplace_back(gamma_out[i], gamma_out[i] + b->hs[i]->ncell);
+            if (heat_out && heat_out[i]) spans.emplace_back(heat_out[i], heat_out[i] + b->hs[i]->ncell);
+        }
+    } catch (const std::bad_alloc&) {
+        return bfail(b, RT_ENOMEM, "out of host memory");
+    }
+    std::sort(spans.begin(), spans.end());
+    bool apart = true;
+    for (size_t k = 1; k < spans.size(); ++k) apart = apart && spans[k - 1].second <= spans[k].first;
+    for (size_t i = 0; i < b->hs.size(); ++i) {
+        const rt_handle* h = b->hs[i];
+        double* const go = gamma_out ? gamma_out[i] : nullptr;
+        double* const ho = heat_out ? heat_out[i] : nullptr;
+        const bool direct = where == RT_DEVICE && apart;
+        b->h_outs[i].gamma = go && direct && direct_access(h, go) ? go : nullptr;
+        b->h_outs[i].heat = ho ? (direct && direct_access(h, ho) ? ho : h->d_heat) : nullptr;
+    }
     float ms = 0.f;
     int rc = run_once(b, &ms);
+    std::copy(b->h_outs, b->h_outs + b->hs.size(), outs.begin());
+    for (size_t i = 0; i < b->hs.size(); ++i) b->h_outs[i] = {nullptr, b->hs[i]->d_heat};   // the buffers are this call's
     if (rc) return rc;
     const cudaMemcpyKind k = where == RT_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
     for (size_t i = 0; i < b->hs.size(); ++i) {
         rt_handle* h = b->hs[i];
+        const FieldOut& o = outs[i];
         const size_t fb = sizeof(double) * (size_t)h->ncell;
-        if (gamma_out && gamma_out[i]) B_CUDA(b, cudaMemcpyAsync(gamma_out[i], h->d_gamma, fb, k, b->stream), "gamma copy");
-        if (heat_out && heat_out[i]) B_CUDA(b, cudaMemcpyAsync(heat_out[i], h->d_heat, fb, k, b->stream), "heat copy");
+        if (gamma_out && gamma_out[i] && !o.gamma)
+            B_CUDA(b, cudaMemcpyAsync(gamma_out[i], h->d_gamma, fb, k, b->stream), "gamma copy");
+        if (heat_out && heat_out[i] && o.heat == h->d_heat)
+            B_CUDA(b, cudaMemcpyAsync(heat_out[i], h->d_heat, fb, k, b->stream), "heat copy");
     }
     B_CUDA(b, cudaStreamSynchronize(b->stream), "output copy");
     if (stats)

@@ -170,23 +170,22 @@ __device__ __forceinline__ void prepare_cells(const FieldJob& J, const int64_t f
 }
 
 // heat = e_heat Gamma n_HI; deposited photons = sum Gamma n_HI dx^3; Gamma copied out (gamma_out null:
-// not). Most cells of an opaque box have no Gamma: a warp without any reads neither field.
+// not). Most cells of an opaque box have no Gamma: a thread without any in its four reads neither field, a
+// warp without any takes no FP64 operation (a test per cell cost more than it saved: 32 against 17 us).
 __device__ __forceinline__ void finalize_cells(const FieldJob& J, const int64_t first, const int64_t stride)
 {
     double dep = 0.0;
     const double heat0 = J.e_heat * 0.0;          // of a cell without Gamma (n_HI is finite)
     for (int64_t t0 = first * kTile; t0 < J.ncell; t0 += stride * kTile) {
-        double g[kUnroll];
+        double g[kUnroll], h[kUnroll];
         bool any = false;
 #pragma unroll
         for (int u = 0; u < kUnroll; ++u) {
             const int64_t c = t0 + u * kBlock + threadIdx.x;
             g[u] = c < J.ncell ? J.gamma[c] : 0.0;
+            h[u] = heat0;
             any = any || bits_of(g[u]) << 1;
         }
-        double h[kUnroll];
-#pragma unroll
-        for (int u = 0; u < kUnroll; ++u) h[u] = heat0;
         if (any) {
             double a[kUnroll], b[kUnroll];
 #pragma unroll
@@ -210,8 +209,9 @@ __device__ __forceinline__ void finalize_cells(const FieldJob& J, const int64_t 
             if (J.heat) J.heat[c] = h[u];
         }
     }
+    if (!__syncthreads_or(bits_of(dep) << 1 != 0)) return;
     dep = block_sum(dep);
-    if (threadIdx.x == 0 && bits_of(dep) << 1) atomicAdd(&J.st->deposited, dep * J.vol);
+    if (threadIdx.x == 0) atomicAdd(&J.st->deposited, dep * J.vol);
 }
 
 template <class R>
@@ -247,10 +247,13 @@ __global__ void __launch_bounds__(kBlock) prepare_many_kernel(const FieldJob* __
     prepare_cells<R>(J, blockIdx.x - J.block0, jobs[j + 1].block0 - J.block0);
 }
 
-__global__ void __launch_bounds__(kBlock) finalize_many_kernel(const FieldJob* __restrict__ jobs, int njobs)
+__global__ void __launch_bounds__(kBlock) finalize_many_kernel(const FieldJob* __restrict__ jobs,
+                                                               const FieldOut* __restrict__ outs, int njobs)
 {
     const int j = job_of_block(jobs, njobs);
-    const FieldJob J = jobs[j];
+    FieldJob J = jobs[j];
+    J.gamma_out = outs[j].gamma;
+    J.heat = outs[j].heat;
     finalize_cells(J, blockIdx.x - J.block0, jobs[j + 1].block0 - J.block0);
 }
 
@@ -314,7 +317,8 @@ int launch_finalize(const FieldJob& j, cudaStream_t s)
     return 1;
 }
 
-uint32_t field_blocks(int64_t ncell) { return (uint32_t)tiles_for(ncell); }
+// Four tiles a block: finding the job costs a block several dependent loads.
+uint32_t field_blocks(int64_t ncell) { return (uint32_t)std::max<int64_t>(1, (ncell + 4 * kTile - 1) / (4 * kTile)); }
 
 int launch_prepare_many(const FieldJob* jobs, int njobs, uint32_t blocks, bool fp32, cudaStream_t s)
 {
@@ -324,10 +328,10 @@ int launch_prepare_many(const FieldJob* jobs, int njobs, uint32_t blocks, bool f
     return 1;
 }
 
-int launch_finalize_many(const FieldJob* jobs, int njobs, uint32_t blocks, cudaStream_t s)
+int launch_finalize_many(const FieldJob* jobs, const FieldOut* outs, int njobs, uint32_t blocks, cudaStream_t s)
 {
     if (njobs <= 0) return 0;
-    finalize_many_kernel<<<blocks, kBlock, 0, s>>>(jobs, njobs);
+    finalize_many_kernel<<<blocks, kBlock, 0, s>>>(jobs, outs, njobs);
     return 1;
 }
 

@@ -1660,61 +1660,51 @@ __device__ __forceinline__ void load_ray(int l, long long j, const RayBuf<R>& in
 }
 
 // Sum a tally over the warp lanes in `mask` that carry the same solve, and add
-// it into that solve's statistics (one atomic per group and counter).
+// it into that solve's statistics (one atomic per group and counter). The whole warp arrives here; the
+// photon sums are trees over it, the other lanes counting zero (an FP64 instruction is 64 cycles, and a
+// sum lane after lane took 96 of them).
 __device__ __forceinline__ void flush_tally(Tally& T, unsigned mask, DevStats* const* st_of_lane, int l)
 {
+    const unsigned all = 0xffffffffu;
     const int lane = threadIdx.x & 31;
-    DevStats* mine = *st_of_lane;
+    DevStats* const mine = *st_of_lane;
     while (mask) {
         const int leader = __ffs(mask) - 1;
-        const unsigned long long key = __shfl_sync(mask, (unsigned long long)mine, leader);
-        const unsigned grp = __ballot_sync(mask, (unsigned long long)mine == key);
-        if ((grp >> lane) & 1u) {
-            const unsigned rays = __reduce_add_sync(grp, T.rays), split = __reduce_add_sync(grp, T.split);
-            const unsigned esc = __reduce_add_sync(grp, T.esc), dtau = __reduce_add_sync(grp, T.dtau);
-            const unsigned dlev = __reduce_add_sync(grp, T.dlev), seg = __reduce_add_sync(grp, T.seg);
-            const unsigned sec = __reduce_add_sync(grp, T.sec);
-            unsigned long long hash = 0ULL;
-            double ab = 0.0, ep = 0.0, dp = 0.0;
-            if (grp == 0xffffffffu) {           // the whole warp: a tree (an FP64 instruction is 64 cycles)
-                hash = T.hash;
-                ab = T.abs;
-                ep = T.escph;
-                dp = T.dropph;
-                for (int o = 16; o > 0; o >>= 1) {
-                    hash += __shfl_xor_sync(grp, hash, o);
-                    ab += __shfl_xor_sync(grp, ab, o);
-                    ep += __shfl_xor_sync(grp, ep, o);
-                    dp += __shfl_xor_sync(grp, dp, o);
-                }
-            } else for (unsigned g = grp; g; g &= g - 1) {
-                const int b = __ffs(g) - 1;
-                hash += __shfl_sync(grp, T.hash, b);
-                ab += __shfl_sync(grp, T.abs, b);
-                ep += __shfl_sync(grp, T.escph, b);
-                dp += __shfl_sync(grp, T.dropph, b);
-            }
-            if (lane == leader && rays) {
-                DevStats* st = mine;
-                atomicAdd(&st->rays[l], (unsigned long long)rays);
-                if (split) atomicAdd(&st->splits[l], (unsigned long long)split);
-                if (esc) atomicAdd(&st->escaped[l], (unsigned long long)esc);
-                if (dtau) atomicAdd(&st->dropped_tau[l], (unsigned long long)dtau);
-                if (dlev) atomicAdd(&st->dropped_level[l], (unsigned long long)dlev);
-                atomicAdd(&st->segments[l], (unsigned long long)seg);
-                if (sec) atomicAdd(&st->secondary[l], (unsigned long long)sec);
-                if (hash) atomicAdd(&st->visit_hash, hash);
-                atomicAdd(&st->absorbed, ab);
-                atomicAdd(&st->escaped_ph, ep);
-                atomicAdd(&st->dropped_ph, dp);
-            }
-            T.clear();
+        const unsigned long long key = __shfl_sync(all, (unsigned long long)mine, leader);
+        const bool in = ((mask >> lane) & 1u) && (unsigned long long)mine == key;
+        const unsigned grp = __ballot_sync(all, in);
+        const unsigned rays = __reduce_add_sync(all, in ? T.rays : 0u), split = __reduce_add_sync(all, in ? T.split : 0u);
+        const unsigned esc = __reduce_add_sync(all, in ? T.esc : 0u), dtau = __reduce_add_sync(all, in ? T.dtau : 0u);
+        const unsigned dlev = __reduce_add_sync(all, in ? T.dlev : 0u), seg = __reduce_add_sync(all, in ? T.seg : 0u);
+        const unsigned sec = __reduce_add_sync(all, in ? T.sec : 0u);
+        unsigned long long hash = in ? T.hash : 0ULL;
+        double ab = in ? T.abs : 0.0, ep = in ? T.escph : 0.0, dp = in ? T.dropph : 0.0;
+        for (int o = 16; o > 0; o >>= 1) {
+            hash += __shfl_xor_sync(all, hash, o);
+            ab += __shfl_xor_sync(all, ab, o);
+            ep += __shfl_xor_sync(all, ep, o);
+            dp += __shfl_xor_sync(all, dp, o);
         }
+        if (lane == leader && rays) {
+            DevStats* st = mine;
+            atomicAdd(&st->rays[l], (unsigned long long)rays);
+            if (split) atomicAdd(&st->splits[l], (unsigned long long)split);
+            if (esc) atomicAdd(&st->escaped[l], (unsigned long long)esc);
+            if (dtau) atomicAdd(&st->dropped_tau[l], (unsigned long long)dtau);
+            if (dlev) atomicAdd(&st->dropped_level[l], (unsigned long long)dlev);
+            atomicAdd(&st->segments[l], (unsigned long long)seg);
+            if (sec) atomicAdd(&st->secondary[l], (unsigned long long)sec);
+            if (hash) atomicAdd(&st->visit_hash, hash);
+            atomicAdd(&st->absorbed, ab);
+            atomicAdd(&st->escaped_ph, ep);
+            atomicAdd(&st->dropped_ph, dp);
+        }
+        if (in) T.clear();
         mask &= ~grp;
     }
 }
 
-// The tallies of a block of kBlock threads, all of one solve, summed and added to its statistics: one
+// The tallies of a block of kLevelBlock threads, all of one solve, summed and added to its statistics: one
 // atomic per block and counter, and none from a block without rays. The three photon sums fold in shared
 // memory, 26 FP64 warp instructions a block; one warp's sums lane after lane took 96, so that a full grid
 // spent 75 us of FP64 pipe on them, whatever it had marched. ph: 3 kLevelBlock doubles of shared memory

@@ -168,6 +168,8 @@ bool geometry_level(int device, long long rq, int level, int n, long long rs, co
 int spectrum_table(int device, double t_bb, SpecTable<double>* d, SpecTable<float>* f, std::string& why);
 // The field check of a handle, enqueued if its fields have not been checked yet.
 int enqueue_field_check(rt_handle* h);
+// Whether a kernel on the handle's device may read or write the caller's buffer p itself.
+bool direct_access(const rt_handle* h, const void* p);
 // The job of a handle's per-cell passes (x: the ionized fraction to use).
 FieldJob field_job(const rt_handle* h, const double* x);
 int handle_prepare_sources(rt_handle* h);

@@ -85,6 +85,12 @@ struct FieldJob {
     uint32_t block0 = 0;
 };
 
+// Where one solve of a batch run leaves its results (either may be null).
+struct FieldOut {
+    double* gamma = nullptr;
+    double* heat = nullptr;
+};
+
 enum : unsigned {
     kErrRayOverflow = 1u,            // next-level ray buffer too small
     kErrUnionFind = 2u,              // union-find retry cap reached
@@ -218,7 +224,8 @@ int launch_finalize(const FieldJob& j, cudaStream_t s);
 // jobs[njobs].block0 = blocks.
 uint32_t field_blocks(int64_t ncell);
 int launch_prepare_many(const FieldJob* jobs, int njobs, uint32_t blocks, bool fp32, cudaStream_t s);
-int launch_finalize_many(const FieldJob* jobs, int njobs, uint32_t blocks, cudaStream_t s);
+// outs[i] replaces jobs[i].gamma_out and heat.
+int launch_finalize_many(const FieldJob* jobs, const FieldOut* outs, int njobs, uint32_t blocks, cudaStream_t s);
 int launch_chem_update(const double* nh, const double* x0, const double* xavg, double* xnew, double* xend,
                        const double* gamma, int64_t ncell, double dt, double alpha_B, double C_H, double clump,
                        DevStats* st, cudaStream_t s);
