@@ -318,12 +318,12 @@ def rt_batch_destroy(b: int) -> None:
     lib().rt_batch_destroy(b)
 
 
+# field names of rt_stats by kind, so that a conversion (one per solve of every run) asks nothing again
+_STATS_FIELDS = [(name, issubclass(kind, C.Array)) for name, kind in rt_stats._fields_]
+
+
 def stats_dict(st: rt_stats) -> dict:
-    out = {}
-    for name, _ in rt_stats._fields_:
-        v = getattr(st, name)
-        out[name] = list(v) if hasattr(v, "__len__") else v
-    return out
+    return {name: getattr(st, name)[:] if is_array else getattr(st, name) for name, is_array in _STATS_FIELDS}
 
 
 # ------------------------------------------------------------ convenience wrapper
