@@ -1924,6 +1924,8 @@ __global__ void __launch_bounds__(256, (kTable && kSingle) ? TableOccupancy<R>::
         }
         __syncthreads();
     }
+    const long long nwarp = (long long)gridDim.x * (blockDim.x >> 5);
+    const long long first_tile = (long long)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
     int lev[RT_MAX_LEVELS + 1];
     long long tot[RT_MAX_LEVELS + 1], nxt[RT_MAX_LEVELS + 1];
     int depth = 0;
@@ -1948,12 +1950,12 @@ __global__ void __launch_bounds__(256, (kTable && kSingle) ? TableOccupancy<R>::
         Tally T;
         T.clear();
         DevStats* cur = nullptr;
-        for (;;) {
-            long long t = 0;
-            if (lane == 0) t = (long long)atomicAdd(&A.tiles[sid], 1ULL);
-            t = __shfl_sync(0xffffffffu, t, 0);
+        // a warp's first tile is its own (consecutive tiles on different SMs); more are claimed only where
+        // there are more tiles than warps, so a small slice, whose level would otherwise wait for every
+        // warp's turn at the counter, takes no atomic
+        const long long ntile = (c1 - c0 + A.tile - 1) / A.tile;
+        for (long long t = first_tile; t < ntile;) {
             const long long s0 = c0 + t * A.tile;
-            if (s0 >= c1) break;
             const long long s1 = min(c1, s0 + (long long)A.tile);
             for (long long base = s0; base < s1; base += 32) {
                 const long long j = base + lane;
@@ -2002,6 +2004,9 @@ __global__ void __launch_bounds__(256, (kTable && kSingle) ? TableOccupancy<R>::
                 }
                 append_split<R>(split, si, pix, oP, otau, ocP, octau, A.buf[l + 1], &A.counts[sid], A.err);
             }
+            if (ntile <= nwarp) break;
+            if (lane == 0) t = nwarp + (long long)atomicAdd(&A.tiles[sid], 1ULL);
+            t = __shfl_sync(0xffffffffu, t, 0);
         }
         const unsigned have = __ballot_sync(0xffffffffu, cur != nullptr);
         if (have) flush_tally(T, have, &cur, l);

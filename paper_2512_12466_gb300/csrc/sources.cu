@@ -244,14 +244,17 @@ __global__ void __launch_bounds__(kBlock) sort_place_kernel(const uint64_t* __re
     __syncthreads();
     const int64_t c0 = blockIdx.x * (int64_t)kSortTile + w * kSortChunk;
     uint64_t k[kSortChunk / 32];
+    int32_t x[kSortChunk / 32];
 #pragma unroll
     for (int u = 0; u < kSortChunk / 32; ++u) {
         const int64_t i = c0 + 32 * u + lane;
         k[u] = i < m ? keys[i] : 0ULL;
+        x[u] = i < m ? (idx ? idx[i] : (int32_t)i) : 0;
         if (i < m) atomicAdd(&slot[w][(int)(k[u] >> shift) & 255], 1);
     }
     // digit t: its count in all tiles and in those before this one
     int all = 0, before = 0;
+#pragma unroll 8
     for (int q = 0; q < (int)gridDim.x; ++q) {
         const int v = hist[q * 256 + t];
         all += v;
@@ -280,7 +283,7 @@ __global__ void __launch_bounds__(kBlock) sort_place_kernel(const uint64_t* __re
         if (v) {
             const int32_t dst = slot[w][d] + __popc(peers & ((1u << lane) - 1u));
             keys_out[dst] = k[u];
-            idx_out[dst] = idx ? idx[i] : (int32_t)i;
+            idx_out[dst] = x[u];
         }
         __syncwarp();
         if (v && (peers >> lane) == 1u) slot[w][d] += __popc(peers);   // the highest lane of its digit
