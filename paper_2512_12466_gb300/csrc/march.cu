@@ -1373,6 +1373,28 @@ __device__ __forceinline__ dflt lin_psi_df(const SpecTable<double>& S, const dou
     return df_add(dflt{a.x, a.y}, df_mul(t, c));
 }
 
+// An opaque segment (dtau >= 2) of a ray with budget Q: the photons it absorbs aQ, their rate before the
+// shares wd = aQ / kap, and the budget left. Not inlined: a thin box never calls it, and inlined its
+// registers cost that march 2%.
+struct OpaqueSeg {
+    double aQ, wd;
+    dflt Q;
+};
+__device__ __noinline__ OpaqueSeg opaque_segment(const float* __restrict__ rtab, const dflt Q, const double dtau,
+                                                 const double kap)
+{
+    // in FP64, where most of the budget goes at once, but without the exponential and the division of
+    // that unit: some fifteen operations (64 cycles of its pipe each) instead of about sixty. The
+    // 64^3 Stromgren step (neutral gas, Delta tau up to 3.5): 4.33 -> 3.63 ms.
+    const double ed = Ieee<double>::lt(dtau, 64.0) ? df_to_double(exp_minus(rtab, df_of(dtau)), 0) : 0.0;
+    const double Qd = df_to_double(Q, 0);
+    OpaqueSeg o;
+    o.aQ = Qd * (1.0 - ed);
+    o.wd = quot_pos(o.aQ, kap);
+    o.Q = df_of(Qd * ed);
+    return o;
+}
+
 // march_ray_table for FP64 physics, in double-float arithmetic as described above. kFreq: Eq. 1 over
 // the blackbody spectrum; Q = P m_G 2^64 then stays the ray's geometric share (its photons are
 // P Phi(tau)), and a segment deposits Q 2^64 r 2^(e_G - 128), r its rate per unit budget and G from
@@ -1514,14 +1536,10 @@ __device__ __forceinline__ bool march_ray_table_df(const SolveView<double>& V, c
                 w = df_mul(Q, dsf);                       // optically thin limit
             }
         } else {
-            // in FP64, where most of the budget goes at once, but without the exponential and the division of
-            // that unit: some fifteen operations (64 cycles of its pipe each) instead of about sixty. The
-            // 64^3 Stromgren step (neutral gas, Delta tau up to 3.5): 4.33 -> 3.63 ms.
-            const double ed = I::lt(dtau, 64.0) ? df_to_double(exp_minus(rtab, df_of(dtau)), 0) : 0.0;
-            const double Qd = df_to_double(Q, 0);
-            aQ = Qd * (1.0 - ed);
-            wd = quot_pos(aQ, kap);
-            Q = df_of(Qd * ed);
+            const OpaqueSeg o = opaque_segment(rtab, Q, dtau, kap);
+            aQ = o.aQ;
+            wd = o.wd;
+            Q = o.Q;
         }
         // ---- Eqs. 5-8: the cell's deposit and the neighbour's
         double dep = 0.0, dep2 = 0.0;
