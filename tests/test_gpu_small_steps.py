@@ -107,6 +107,30 @@ def test_bubble_radii(nyx, dr, rmax, periodic):
     s.close()
 
 
+def test_sort_of_many_tiles(nyx):
+    # more tiles than the sort has blocks (512 of 1024 keys): several tiles a block
+    m = 600 * 1024 + 77
+    rng = np.random.default_rng(31)
+    w = I.random_small(64, 1, seed=950, x_mode="neutral", box_cm=64 * 3e21)
+    cells, rates = rng.integers(0, 64, size=(m, 3)).astype(np.int32), rng.uniform(1, 2, m) * 1e48
+    s = nyx.Solver(w.n, w.box_cm, n_th_cm3=1e-6)
+    s.set_fields(dev(w.n_h, np.float64), dev(w.x_ion, np.float64))
+    s.add_sources(dev(cells, np.int32), dev(rates, np.float64))
+    s.step(0.0, torch.empty(w.n ** 3, dtype=torch.float64, device="cuda"), None)
+    key = (cells[:, 0].astype(np.int64) * 64 + cells[:, 1]) * 64 + cells[:, 2]
+    order = np.argsort(key, kind="stable")
+    uniq, start = np.unique(key[order], return_index=True)
+    got_c, got_r = s.sources()
+    assert np.array_equal((got_c[:, 0].astype(np.int64) * 64 + got_c[:, 1]) * 64 + got_c[:, 2], uniq)
+    for u in rng.integers(0, len(uniq), 2000):                   # sums in input order, bit for bit
+        run = rates[order[start[u]: start[u + 1] if u + 1 < len(start) else m]]
+        acc = run[0]
+        for v in run[1:]:
+            acc = acc + v
+        assert got_r[u] == acc
+    s.close()
+
+
 @pytest.mark.parametrize("dx", [3e20, 2e21, 5e22, 7e23])
 def test_opaque_segments_fp64(nyx, dx):
     # optical depths per segment from thin through the switch at 2 to far beyond (neutral gas)
