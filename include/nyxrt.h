@@ -144,8 +144,8 @@ typedef struct rt_stats {
     double chem_residual;      /* last max |<x>_new - <x>_old| */
     double ms_trace;           /* device time of the last trace, first to last march launch */
     double ms_step;            /* device time of the whole step */
-    double ms_march;           /* sum of the march kernels' own durations in the last trace
-                                  (CUDA events around each launch, on the handle's stream) */
+    double ms_march;           /* the same as ms_trace: from the first march launch of the last trace to
+                                  the end of its last (levels are launched one behind the other) */
     int64_t march_launches;    /* march kernel launches in the last trace */
     int64_t table_levels;      /* bit l set: level l's march read its cells from the per-device
                                   geometry tables in the last trace; clear: it walked its rays

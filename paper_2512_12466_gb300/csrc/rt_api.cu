@@ -6,8 +6,8 @@
 // tracing loop of Alg. 2 as one fused march+split launch per level (and per
 // slice when a level's rays exceed the per-launch bound), then the heating
 // and ledger reduction; with chemistry it iterates trace and the C2-Ray
-// update (Sec. 2.4). The host reads back one counter per launch to size the
-// next level; everything else stays on the device.
+// update (Sec. 2.4). Levels of bounded size follow each other without the host (their counts stay on the
+// device); above that it reads one counter to size the next.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -1432,7 +1432,7 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
     h->launches += launch_finalize(job, s);
     RT_LAUNCHED(h, "finalize launch");
     if (h->cfg.chem_iterate) {
-        std::swap(h->d_x, h->d_xend);         // x(t + dt)
+        RT_CUDA(h, cudaMemcpyAsync(h->d_x, h->d_xend, fb, cudaMemcpyDeviceToDevice, s), "x update");   // x(t + dt)
         h->fields_checked = false;
     }
     const cudaMemcpyKind k = where == RT_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
