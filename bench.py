@@ -48,9 +48,9 @@ L2_FLUSH_BYTES = 512 << 20
 # [--precision fp64]`), scaled to the full workload by primary segments. Valid only for the kernel
 # sources it was taken on.
 TRAFFIC_CAPTURE = {"kernel": "march_table_kernel",
-                   "bytes_per_segment": {"fp32": 8.80868621095342, "fp64": 19.254816976037528},
-                   "sources": {"paper_2512_12466_gb300/csrc/march.cu": "e97eefbf436b7d8a",
-                               "paper_2512_12466_gb300/csrc/rt_internal.h": "7b899d1021ce1758",
+                   "bytes_per_segment": {"fp32": 8.626376059933783, "fp64": 19.1181517084529},
+                   "sources": {"paper_2512_12466_gb300/csrc/march.cu": "17d4ef3d9baa504b",
+                               "paper_2512_12466_gb300/csrc/rt_internal.h": "d0567305ea6de2d9",
                                "paper_2512_12466_gb300/csrc/dfloat.h": "459135c9d92ee117"}}
 
 
