@@ -119,14 +119,16 @@ __global__ void __launch_bounds__(kBlock) check_fields_kernel(const double* __re
     }
 }
 
-// v >= 0 rounded to the nearest float, ties to even, on the integer pipe: the head's 24 bits and the
-// rest, shifted down first where the result is subnormal.
+// v rounded to the nearest float, ties to even, on the integer pipe: the magnitude's leading 24 bits and
+// the rest, shifted down first where the result is subnormal; the sign is carried over.
 __device__ __forceinline__ float narrow(const double v)
 {
-    const unsigned hi = (unsigned)(bits_of(v) >> 32), lo = (unsigned)bits_of(v);
+    const unsigned sign = (unsigned)(bits_of(v) >> 32) & 0x80000000u;
+    const unsigned hi = (unsigned)(bits_of(v) >> 32) & 0x7fffffffu, lo = (unsigned)bits_of(v);
     unsigned u = ((hi - 0x38000000u) << 3) | (lo >> 29), rem = lo << 3;       // rem: in units of 2^-32 of u's last place
     if (hi - 0x38100000u >= 0x47f00000u - 0x38100000u) {                      // not a normal float (zero among them)
-        if (hi >= 0x47f00000u) return __uint_as_float(hi > 0x7ff00000u || (hi == 0x7ff00000u && lo) ? 0x7fffffffu : 0x7f800000u);
+        if (hi >= 0x47f00000u)
+            return __uint_as_float(sign | (hi > 0x7ff00000u || (hi == 0x7ff00000u && lo) ? 0x7fffffffu : 0x7f800000u));
         const int down = 897 - (int)(hi >> 20);                               // 1 .. 897
         const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
         const unsigned long long w = down < 32 ? m >> down : 0ull;            // below 2^-158: nothing
@@ -135,7 +137,16 @@ __device__ __forceinline__ float narrow(const double v)
         rem = ((unsigned)w << 3) | (sticky ? 1u : 0u);
     }
     u += (rem > 0x80000000u || (rem == 0x80000000u && (u & 1u))) ? 1u : 0u;
-    return __uint_as_float(u);
+    return __uint_as_float(sign | u);
+}
+
+// k where the cell may receive a secondary deposit, -k elsewhere, for any sign of k (a -0.0 in n_H gives a
+// negative zero).
+template <class R>
+__device__ __forceinline__ R stored_kappa(const double k, const bool elig)
+{
+    if constexpr (sizeof(R) == 4) return __uint_as_float(__float_as_uint(narrow(k)) ^ (elig ? 0u : 0x80000000u));
+    else return __longlong_as_double(bits_of(k) ^ (elig ? 0ll : (long long)0x8000000000000000ull));
 }
 
 // kappa = (sigma dx) ((1 - x) n_H), the optical depth per cell length, and Gamma cleared.
@@ -163,11 +174,7 @@ __device__ __forceinline__ void prepare_cells(const FieldJob& J, const int64_t f
             const double nhi = __dmul_rn(__dsub_rn(1.0, b[u]), a[u]);
             const double k = __dmul_rn(J.sdx, nhi);
             const bool elig = bits_of(a[u]) >= bits_of(n_th) && bits_of(nhi) > 0;
-            if constexpr (sizeof(R) == 4) {
-                kap[c] = __uint_as_float(__float_as_uint(narrow(k)) | (elig ? 0u : 0x80000000u));
-            } else {
-                kap[c] = __longlong_as_double(bits_of(k) | (elig ? 0ll : (long long)0x8000000000000000ull));
-            }
+            kap[c] = stored_kappa<R>(k, elig);
             J.gamma[c] = 0.0;
         }
     }
