@@ -140,6 +140,20 @@ __device__ __forceinline__ float narrow(const double v)
     return __uint_as_float(sign | u);
 }
 
+// n_th's place in the order of bit patterns; above every density where it is a NaN of either sign (no cell
+// is eligible then, as none compares >= to it).
+__device__ __forceinline__ long long threshold_bits(const double n_th)
+{
+    const long long b = bits_of(n_th);
+    return (b & 0x7fffffffffffffffll) > 0x7ff0000000000000ll ? 0x7fffffffffffffffll : b;
+}
+
+// Eqs. 7-8: whether a cell may receive a secondary deposit, n_H >= n_th and n_HI > 0.
+__device__ __forceinline__ bool eligible(const double nh, const double nhi, const long long th)
+{
+    return bits_of(nh) >= th && bits_of(nhi) > 0;
+}
+
 // k where the cell may receive a secondary deposit, -k elsewhere, for any sign of k (a -0.0 in n_H gives a
 // negative zero).
 template <class R>
@@ -157,7 +171,7 @@ __device__ __forceinline__ R stored_kappa(const double k, const bool elig)
 template <class R>
 __device__ __forceinline__ void prepare_cells(const FieldJob& J, const int64_t first, const int64_t stride)
 {
-    const double n_th = J.chk ? J.chk->n_th : J.n_th;
+    const long long th = threshold_bits(J.chk ? J.chk->n_th : J.n_th);
     R* const kap = static_cast<R*>(J.kap);
     for (int64_t t0 = first * kTile; t0 < J.ncell; t0 += stride * kTile) {
         double a[kUnroll], b[kUnroll];
@@ -173,8 +187,7 @@ __device__ __forceinline__ void prepare_cells(const FieldJob& J, const int64_t f
             if (c >= J.ncell) break;
             const double nhi = __dmul_rn(__dsub_rn(1.0, b[u]), a[u]);
             const double k = __dmul_rn(J.sdx, nhi);
-            const bool elig = bits_of(a[u]) >= bits_of(n_th) && bits_of(nhi) > 0;
-            kap[c] = stored_kappa<R>(k, elig);
+            kap[c] = stored_kappa<R>(k, eligible(a[u], nhi, th));
             J.gamma[c] = 0.0;
         }
     }

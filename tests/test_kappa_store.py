@@ -13,10 +13,13 @@ def dev(tmp_path_factory):
     src = source("fields.cu")
     body = "".join(definition(src, s) for s in ("__device__ __forceinline__ long long bits_of(",
                                                 "__device__ __forceinline__ float narrow(",
-                                                "__device__ __forceinline__ R stored_kappa("))
+                                                "__device__ __forceinline__ R stored_kappa(",
+                                                "__device__ __forceinline__ long long threshold_bits(",
+                                                "__device__ __forceinline__ bool eligible("))
     return compile_host(tmp_path_factory.mktemp("kappa"), body + """
 extern "C" void f32(const double* k, int n, int elig, float* out) { for (int i = 0; i < n; ++i) out[i] = stored_kappa<float>(k[i], elig); }
 extern "C" void f64(const double* k, int n, int elig, double* out) { for (int i = 0; i < n; ++i) out[i] = stored_kappa<double>(k[i], elig); }
+extern "C" int elig(double nh, double x, double n_th) { return eligible(nh, (1.0 - x) * nh, threshold_bits(n_th)); }
 """)
 
 
@@ -38,3 +41,12 @@ def test_stored_kappa_is_the_rounded_signed_value(dev, elig):
         want32 = want.astype(np.float32)
     assert np.array_equal(run(dev, "f32", np.float32, k, elig).view(np.uint32), want32.view(np.uint32))
     assert np.array_equal(run(dev, "f64", np.float64, k, elig).view(np.uint64), want.view(np.uint64))
+
+
+def test_eligible_is_the_comparison(dev):
+    # valid densities and fractions, both zeros, against every kind of threshold, NaNs of both signs among them
+    dev.elig.argtypes = [C.c_double] * 3
+    for n_th in (0.0, -0.0, 5e-324, 1e-6, 1.0, np.inf, np.nan, np.copysign(np.nan, -1.0)):
+        for nh in (0.0, -0.0, 5e-324, 1e-6, np.nextafter(1e-6, 0), 1.0, 1e300):
+            for x in (0.0, -0.0, 0.5, 1.0):
+                assert bool(dev.elig(nh, x, n_th)) == (nh >= n_th and (1.0 - x) * nh > 0.0), (nh, x, n_th)
