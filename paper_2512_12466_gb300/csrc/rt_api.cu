@@ -745,12 +745,24 @@ FieldJob field_job(const rt_handle* h, const double* x)
 int enqueue_field_check(rt_handle* h)
 {
     const bool want_x = h->cfg.merge_mode == RT_MERGE_AUTO;
-    if (h->fields_checked && (h->checked_x || !want_x)) return RT_OK;
+    if (h->fields_checked && !h->fields_recorded && (h->checked_x || !want_x)) return RT_OK;
     h->launches += launch_check_fields(h->d_nh, h->d_x, h->ncell, nullptr, nullptr, want_x, h->d_chk, h->stream);
     RT_LAUNCHED(h, "check launch");
     h->fields_checked = true;
     h->checked_x = want_x;
     return RT_OK;
+}
+
+// Whether the handle's stream is being captured into a graph (the default stream never is).
+static bool capturing(const rt_handle* h)
+{
+    if (h->stream == nullptr || h->stream == cudaStreamLegacy) return false;
+    cudaStreamCaptureStatus st = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(h->stream, &st) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return st != cudaStreamCaptureStatusNone;
 }
 
 // A caller's buffer that a kernel on the handle's device may read or write itself: aligned memory of
@@ -1126,6 +1138,7 @@ int rt_set_fields(rt_handle* h, const double* n_H, const double* x_ion, int wher
     DeviceGuard g(h->device);
     const size_t fb = sizeof(double) * (size_t)h->ncell;
     h->fields_checked = false;
+    if (capturing(h)) h->fields_recorded = true;
     if (where == RT_DEVICE && direct_access(h, n_H) && direct_access(h, x_ion)) {
         // copied and checked in one pass
         const bool want_x = h->cfg.merge_mode == RT_MERGE_AUTO;

@@ -108,6 +108,8 @@ struct rt_handle {
     nyx::FieldCheck* d_chk = nullptr;     // of d_nh and d_x, while fields_checked
     bool fields_checked = false;          // the check has run (or is enqueued) on the fields as they are
     bool checked_x = false;               // with the sum of x
+    bool fields_recorded = false;         // an rt_set_fields is in a caller's graph: the fields may change
+                                          // unseen, so no check outlasts a call
 
     nyx::SourceWork sw;
     int64_t nsrc = 0;
