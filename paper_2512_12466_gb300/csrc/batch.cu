@@ -43,6 +43,14 @@ __global__ void tag_sources_kernel(const SrcEntry* __restrict__ in, int64_t m, i
     }
 }
 
+// The heavy solves' error words (each launch has its solve's) into the run's, which the writing of results
+// asks.
+__global__ void fold_errors_kernel(const DevStats* __restrict__ st, int count, unsigned* err)
+{
+    for (int i = threadIdx.x; i < count; i += blockDim.x)
+        if (st[i].err) atomicOr(err, st[i].err);
+}
+
 constexpr int kMaxSlices = 1 << 16;
 // Heavy solves: lanes, and the ray-record bytes one lane's chunk may need at most (a chunk holds as
 // many sources as keep every level's parent records within it).
@@ -403,8 +411,11 @@ int enqueue(rt_batch* b)
     if (any_heavy) {
         const int rc = enqueue_heavy(b, hv);
         if (rc) return rc;
+        fold_errors_kernel<<<1, 256, 0, s>>>(b->d_stats, (int)b->hs.size(), b->d_err);
+        B_CUDA(b, cudaGetLastError(), "error launch");
+        b->launches += 1;
     }
-    b->launches += launch_finalize_many(b->d_jobs, b->d_outs, (int)b->hs.size(), b->field_blocks, s);
+    b->launches += launch_finalize_many(b->d_jobs, b->d_outs, b->d_err, (int)b->hs.size(), b->field_blocks, s);
     B_CUDA(b, cudaGetLastError(), "finalize launch");
     // statistics and error word written into pinned memory by a kernel, not copied: a server's
     // result copies of the previous batch may occupy the copy engines
@@ -478,9 +489,9 @@ int run_launch(rt_batch* b)
 int run_finish(rt_batch* b, float* ms)
 {
     B_CUDA(b, cudaStreamSynchronize(b->stream), "batch run");
-    if (*b->h_err) return bfail(b, RT_EDEVICE, "batch kernel reported an internal error (buffer, slice or level limit)");
     for (size_t i = 0; i < b->hs.size(); ++i)
         if (b->h_stats[i].err) return bfail(b, RT_EDEVICE, "a march launch of a heavy solve reported an internal error");
+    if (*b->h_err) return bfail(b, RT_EDEVICE, "batch kernel reported an internal error (buffer, slice or level limit)");
     if (ms) B_CUDA(b, cudaEventElapsedTime(ms, b->ev0, b->ev1), "event");
     b->work.assign(b->hs.size(), 0ULL);           // the next launches' grouping (a graph keeps its own)
     for (size_t i = 0; i < b->hs.size(); ++i)

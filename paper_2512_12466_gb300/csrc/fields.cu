@@ -247,7 +247,8 @@ __global__ void __launch_bounds__(kBlock) prepare_kappa_kernel(const FieldJob J)
 
 __global__ void __launch_bounds__(kBlock) finalize_kernel(const FieldJob J)
 {
-    if (J.valid && J.st->bad_input) return;
+    // nothing goes to the caller's arrays from inputs found invalid or from a trace that reported an error
+    if (J.valid && (J.st->bad_input || J.st->err)) return;
     finalize_cells(J, blockIdx.x, gridDim.x);
 }
 
@@ -272,8 +273,10 @@ __global__ void __launch_bounds__(kBlock) prepare_many_kernel(const FieldJob* __
 }
 
 __global__ void __launch_bounds__(kBlock) finalize_many_kernel(const FieldJob* __restrict__ jobs,
-                                                               const FieldOut* __restrict__ outs, int njobs)
+                                                               const FieldOut* __restrict__ outs,
+                                                               const unsigned* err, int njobs)
 {
+    if (*err) return;                             // of any solve: the run fails and no result is written
     const int j = job_of_block(jobs, njobs);
     FieldJob J = jobs[j];
     J.gamma_out = outs[j].gamma;
@@ -352,10 +355,11 @@ int launch_prepare_many(const FieldJob* jobs, int njobs, uint32_t blocks, bool f
     return 1;
 }
 
-int launch_finalize_many(const FieldJob* jobs, const FieldOut* outs, int njobs, uint32_t blocks, cudaStream_t s)
+int launch_finalize_many(const FieldJob* jobs, const FieldOut* outs, const unsigned* err, int njobs, uint32_t blocks,
+                         cudaStream_t s)
 {
     if (njobs <= 0) return 0;
-    finalize_many_kernel<<<blocks, kBlock, 0, s>>>(jobs, outs, njobs);
+    finalize_many_kernel<<<blocks, kBlock, 0, s>>>(jobs, outs, err, njobs);
     return 1;
 }
 

@@ -1450,10 +1450,11 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
     }
     const cudaMemcpyKind k = where == RT_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
     if ((gamma_out && !gamma_direct) || (heat_out && !heat_direct)) {
-        // nothing is copied over the caller's data before the inputs are known to be valid
+        // nothing is copied over the caller's data before the inputs and the trace are known to be sound
         RT_CUDA(h, cudaMemcpyAsync(h->h_words, h->d_words, sizeof(StepWords), cudaMemcpyDeviceToHost, s), "input check");
         RT_CUDA(h, cudaStreamSynchronize(s), "step");
         if (h->h_st->bad_input) return reject(h);
+        if (h->h_st->err) return fail(h, RT_EDEVICE, "a kernel reported an internal error");
     }
     if (gamma_out && !gamma_direct) RT_CUDA(h, cudaMemcpyAsync(gamma_out, h->d_gamma, fb, k, s), "gamma copy");
     if (heat_out && !heat_direct) RT_CUDA(h, cudaMemcpyAsync(heat_out, h->d_heat, fb, k, s), "heat copy");

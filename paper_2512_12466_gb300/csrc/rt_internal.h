@@ -80,7 +80,7 @@ struct FieldJob {
     double e_heat = 0, vol = 0;
     const FieldCheck* chk = nullptr; // given: n_th from there
     const FieldCheck* valid = nullptr; // given: its invalid cells go to st->bad_input before the trace, and
-                                       // where that is not zero no result is written
+                                       // where that or st->err is not zero no result is written
     DevStats* st = nullptr;
     uint32_t block0 = 0;
 };
@@ -224,8 +224,9 @@ int launch_finalize(const FieldJob& j, cudaStream_t s);
 // jobs[njobs].block0 = blocks.
 uint32_t field_blocks(int64_t ncell);
 int launch_prepare_many(const FieldJob* jobs, int njobs, uint32_t blocks, bool fp32, cudaStream_t s);
-// outs[i] replaces jobs[i].gamma_out and heat.
-int launch_finalize_many(const FieldJob* jobs, const FieldOut* outs, int njobs, uint32_t blocks, cudaStream_t s);
+// outs[i] replaces jobs[i].gamma_out and heat; nothing is written where *err is set.
+int launch_finalize_many(const FieldJob* jobs, const FieldOut* outs, const unsigned* err, int njobs, uint32_t blocks,
+                         cudaStream_t s);
 int launch_chem_update(const double* nh, const double* x0, const double* xavg, double* xnew, double* xend,
                        const double* gamma, int64_t ncell, double dt, double alpha_B, double C_H, double clump,
                        DevStats* st, cudaStream_t s);
