@@ -145,21 +145,42 @@ size_t geometry_budget(int device)
     return total_b / 4;
 }
 
+// The smallest table that covers grids of n cells and was built for at most n + n/4: one built for
+// a much larger grid, complete or not, holds rows this grid never reads (level 10 at 1024^3 is
+// 38 GB in FP32, against 10 GB at 256^3), so a grid that small gets its own. Null: none yet.
+GeomTable* geometry_find(std::vector<GeomTable>& list, long long rq, int level, int n, long long rs)
+{
+    GeomTable* t = nullptr;
+    for (GeomTable& c : list)
+        if (c.rq == rq && c.rs == rs && c.level == level && (c.complete || c.n_cover >= n) &&
+            c.n_cover <= n + n / 4 && (!t || c.n_cover < t->n_cover))
+            t = &c;
+    return t;
+}
+
 }  // namespace
+
+nyx::GeomState nyx::geometry_state(int device, long long rq, int level, int n, long long rs, bool fp64, GeomLevel* out)
+{
+    std::lock_guard<std::mutex> lk(g_geom_mu);
+    const GeomTable* t = geometry_find(g_geom[device], rq, level, n, rs);
+    if (!t) return GeomState::unbuilt;
+    if (t->row0 && (fp64 ? t->ent64 != nullptr : t->ent != nullptr)) {
+        out->ent = t->ent;
+        out->ent64 = t->ent64;
+        out->row0 = t->row0;
+        return GeomState::ready;
+    }
+    const size_t failed = !t->row0 ? t->failed_rows : (fp64 ? t->failed64 : t->failed32);
+    return failed == 0 || geometry_budget(device) > failed ? GeomState::unbuilt : GeomState::none;
+}
 
 bool nyx::geometry_level(int device, long long rq, int level, int n, long long rs, const int4* dirs_level,
                          cudaStream_t s, bool fp64, GeomLevel* out)
 {
     std::lock_guard<std::mutex> lk(g_geom_mu);
     std::vector<GeomTable>& list = g_geom[device];
-    // the smallest table that covers grids of n cells and was built for at most n + n/4: one built for
-    // a much larger grid, complete or not, holds rows this grid never reads (level 10 at 1024^3 is
-    // 38 GB in FP32, against 10 GB at 256^3), so a grid that small gets its own
-    GeomTable* t = nullptr;
-    for (GeomTable& c : list)
-        if (c.rq == rq && c.rs == rs && c.level == level && (c.complete || c.n_cover >= n) &&
-            c.n_cover <= n + n / 4 && (!t || c.n_cover < t->n_cover))
-            t = &c;
+    GeomTable* t = geometry_find(list, rq, level, n, rs);
     const long long npix = 12LL << (2 * level);
     const long long nb = (npix + 31) / 32;
     const size_t budget = geometry_budget(device);
@@ -627,8 +648,9 @@ int ensure_rays(rt_handle* h, int level, int64_t need)
 }
 
 // One march launch: children [c0, c1) of `level`, or as many of them as the device counted (counted).
+// ready: the level's geometry table, if it is in place (null: built here, once per device, or walked).
 template <class R>
-int launch_level(rt_handle* h, int level, int64_t c0, int64_t c1, bool counted, bool early)
+int launch_level(rt_handle* h, int level, int64_t c0, int64_t c1, bool counted, bool early, const GeomLevel* ready)
 {
     char range[32];
     std::snprintf(range, sizeof(range), "march level %d", level);
@@ -671,10 +693,11 @@ int launch_level(rt_handle* h, int level, int64_t c0, int64_t c1, bool counted, 
     // grid-stride blocks of equal share: 12 per SM is a whole number of waves for the march
     // kernels' 2, 3 and 4 resident blocks per SM, so no last wave runs an SM part-empty
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)h->sm_count * kMarchBlocksPerSm));
-    // the level's geometry table for this precision (built once per device)
     GeomLevel gl;
-    const bool table = !(h->cfg.flags & RT_FLAG_NO_GEOMETRY_TABLE) &&
-                       geometry_level(h->device, h->rq, level, h->cfg.n, h->rs, a.dirs, h->stream, sizeof(R) == 8, &gl);
+    if (ready) gl = *ready;
+    const bool table = ready || (!(h->cfg.flags & RT_FLAG_NO_GEOMETRY_TABLE) &&
+                                 geometry_level(h->device, h->rq, level, h->cfg.n, h->rs, a.dirs, h->stream,
+                                                sizeof(R) == 8, &gl));
     if constexpr (sizeof(R) == 8) {
         if (table) launch_march_table_f64(a, gl, grid, h->stream);
         else launch_march_f64(a, grid, h->stream);
@@ -691,8 +714,9 @@ int launch_level(rt_handle* h, int level, int64_t c0, int64_t c1, bool counted, 
 
 // March `total` rays of `level` and all that follow from them, one slice of children at a time.
 // A slice's next levels are enqueued behind it while their bound (every ray splits) stays within
-// kChainChildren; the host reads the count of the level after those, if there is one, and goes on from
-// there. counted: `total` is a bound itself (level 0, with the catalog's size on the device).
+// kChainChildren and their geometry tables are in place (or not to be had); the host reads the count of
+// the level after those, if there is one, and goes on from there, so that a table is built only for a
+// level that rays reach (levels 0 to 8 of a box of 128^3 cells or more take 0.7 GB in FP32, 1.4 in FP64). counted: `total` is a bound itself (level 0, with the catalog's size on the device).
 template <class R>
 int run_levels(rt_handle* h, int level, int64_t total, bool counted)
 {
@@ -706,12 +730,17 @@ int run_levels(rt_handle* h, int level, int64_t total, bool counted)
                                        sizeof(unsigned long long) * (size_t)(RT_MAX_LEVELS - level), h->stream), "counters");
         int l = level;
         int64_t bound = c1 - c0;
-        int rc = launch_level<R>(h, l, c0, c1, counted, false);
+        int rc = launch_level<R>(h, l, c0, c1, counted, false, nullptr);
         if (rc) return rc;
         while (l < h->table_level && 4 * bound <= kChainChildren) {
+            GeomLevel gl;
+            GeomState have = GeomState::none;
+            if (!(h->cfg.flags & RT_FLAG_NO_GEOMETRY_TABLE))
+                have = geometry_state(h->device, h->rq, l + 1, h->cfg.n, h->rs, sizeof(R) == 8, &gl);
+            if (have == GeomState::unbuilt) break;
             ++l;
             bound *= 4;
-            rc = launch_level<R>(h, l, 0, bound, true, true);
+            rc = launch_level<R>(h, l, 0, bound, true, true, have == GeomState::ready ? &gl : nullptr);
             if (rc) return rc;
         }
         if (l == h->table_level) continue;
@@ -1498,7 +1527,8 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
         st->ms_step = ms;
         st->ms_march = h->cfg.chem_iterate ? h->ms_march : st->ms_trace;
         st->march_launches = h->march_launches;
-        st->table_levels = h->table_levels;
+        for (int l = 0; l < RT_MAX_LEVELS; ++l)                // a level launched in vain read nothing
+            if (d.rays[l]) st->table_levels |= h->table_levels & (int64_t(1) << l);
     }
     return RT_OK;
 }

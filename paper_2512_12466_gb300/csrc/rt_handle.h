@@ -166,6 +166,9 @@ int ensure_directions(int device, int level, const int4** out, std::string& err)
 // precision (over the device's table budget), so its rays are walked.
 bool geometry_level(int device, long long rq, int level, int n, long long rs, const int4* dirs_level,
                     cudaStream_t s, bool fp64, GeomLevel* out);
+// What geometry_level would find: the table in place (*out is it), none to be had, or one to build first.
+enum class GeomState { ready, none, unbuilt };
+GeomState geometry_state(int device, long long rq, int level, int n, long long rs, bool fp64, GeomLevel* out);
 // The RT_SPECTRUM_BLACKBODY tables at t_bb for `device` (device < 0: host table only).
 int spectrum_table(int device, double t_bb, SpecTable<double>* d, SpecTable<float>* f, std::string& why);
 // The field check of a handle, enqueued if its fields have not been checked yet.
