@@ -164,7 +164,10 @@ void rt_config_default(rt_config* cfg, int32_t n, double box_cm);
 
 /* Create a solver for one grid (Sec. 2.5 ray-tracing state). `cuda_stream`
  * is a cudaStream_t (NULL = legacy default stream) on the current device.
- * Allocates the field and ray buffers on that device. */
+ * Allocates the field buffers on that device; the ray buffers grow in its
+ * steps. Those of levels that can hold at most 2^21 rays are sized for that
+ * bound rather than the rays found (67 MB for the largest), where there is
+ * memory for it. */
 int rt_create(const rt_config* cfg, void* cuda_stream, rt_handle** out);
 
 /* Copy the hydrogen density n_H (cm^-3, >= 0, finite) and the ionized

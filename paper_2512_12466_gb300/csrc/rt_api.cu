@@ -526,7 +526,8 @@ bool valid_config(const rt_config* c, std::string& why);
 
 // Host-side fault injection for tests: with NYXRT_FAULT_ALLOC=k (k >= 1) in the environment, the k-th
 // handle allocation the library makes through dalloc in this process fails as if the device were out
-// of memory (no device work is involved; every caller must return RT_ENOMEM and stay usable). With
+// of memory (no device work is involved; every caller must do without it or return RT_ENOMEM and stay
+// usable). With
 // NYXRT_FAULT_ALLOC_TRACE set, every dalloc call writes its ordinal to stderr ("nyxrt-dalloc k"), so
 // a test can find which ordinals a stage makes before it injects one.
 long long fault_alloc_at()
@@ -631,20 +632,22 @@ int grow_sources(rt_handle* h, int64_t need)
     return RT_OK;
 }
 
+// The level's ray buffer, grown to hold `need` records; a level without one where that fails.
 template <class R>
-int ensure_rays(rt_handle* h, int level, int64_t need)
+cudaError_t grow_rays(rt_handle* h, int level, int64_t need)
 {
     RayStore& s = h->rays[level];
-    if (s.cap >= need) return RT_OK;
+    if (s.cap >= need) return cudaSuccess;
     int64_t cap = std::max<int64_t>(need, std::min<int64_t>(kMaxChildrenPerLaunch, std::max<int64_t>(4096, 2 * s.cap)));
     dfree(h, s.base);
     s.base = nullptr;
     s.cap = 0;
     void* p = nullptr;
-    RT_CUDA(h, dalloc(h, &p, ray_bytes(cap, (int)sizeof(R))), "ray buffer");
+    const cudaError_t e = dalloc(h, &p, ray_bytes(cap, (int)sizeof(R)));
+    if (e != cudaSuccess) return e;
     s.base = p;
     s.cap = cap;
-    return RT_OK;
+    return cudaSuccess;
 }
 
 // One march launch: children [c0, c1) of `level`, or as many of them as the device counted (counted).
@@ -657,10 +660,7 @@ int launch_level(rt_handle* h, int level, int64_t c0, int64_t c1, bool counted, 
     NvtxRange nvtx(range);
     // rays of the deepest level end before their split sphere or at level_max
     const bool can_split = level < h->table_level;
-    if (can_split) {
-        const int rc = ensure_rays<R>(h, level + 1, c1 - c0);
-        if (rc) return rc;
-    }
+    if (can_split) RT_CUDA(h, grow_rays<R>(h, level + 1, c1 - c0), "ray buffer");
     MarchArgs<R> a;
     a.level = level;
     a.n = h->cfg.n;
@@ -714,9 +714,11 @@ int launch_level(rt_handle* h, int level, int64_t c0, int64_t c1, bool counted, 
 
 // March `total` rays of `level` and all that follow from them, one slice of children at a time.
 // A slice's next levels are enqueued behind it while their bound (every ray splits) stays within
-// kChainChildren and their geometry tables are in place (or not to be had); the host reads the count of
-// the level after those, if there is one, and goes on from there, so that a table is built only for a
-// level that rays reach (levels 0 to 8 of a box of 128^3 cells or more take 0.7 GB in FP32, 1.4 in FP64). counted: `total` is a bound itself (level 0, with the catalog's size on the device).
+// kChainChildren, their geometry tables are in place (or not to be had) and there is memory for the rays
+// the bound allows; the host reads the count of the level after those, if there is one, and goes on from
+// there. So a table is built only for a level that rays reach (levels 0 to 8 of a box of 128^3 cells or
+// more take 0.7 GB in FP32, 1.4 in FP64), and a step fails for want of memory only where its rays need it.
+// counted: `total` is a bound itself (level 0, with the catalog's size on the device).
 template <class R>
 int run_levels(rt_handle* h, int level, int64_t total, bool counted)
 {
@@ -738,6 +740,10 @@ int run_levels(rt_handle* h, int level, int64_t total, bool counted)
             if (!(h->cfg.flags & RT_FLAG_NO_GEOMETRY_TABLE))
                 have = geometry_state(h->device, h->rq, l + 1, h->cfg.n, h->rs, sizeof(R) == 8, &gl);
             if (have == GeomState::unbuilt) break;
+            if (l + 1 < h->table_level && grow_rays<R>(h, l + 2, 4 * bound) != cudaSuccess) {
+                cudaGetLastError();          // perhaps enough for the rays there are
+                break;
+            }
             ++l;
             bound *= 4;
             rc = launch_level<R>(h, l, 0, bound, true, true, have == GeomState::ready ? &gl : nullptr);
