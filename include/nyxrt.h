@@ -144,8 +144,10 @@ typedef struct rt_stats {
     double chem_residual;      /* last max |<x>_new - <x>_old| */
     double ms_trace;           /* device time of the last trace, first to last march launch */
     double ms_step;            /* device time of the whole step */
-    double ms_march;           /* the same as ms_trace: from the first march launch of the last trace to
-                                  the end of its last (levels are launched one behind the other) */
+    double ms_march;           /* device time of the last trace's march launches: the sum over the runs of
+                                  launches that follow one another without the host, each from its
+                                  first launch to the end of its last (CUDA events); host waits, table
+                                  builds and the growth of ray buffers are not in it */
     int64_t march_launches;    /* march kernel launches in the last trace */
     int64_t table_levels;      /* bit l set: level l's march read its cells from the per-device
                                   geometry tables in the last trace; clear: it walked its rays

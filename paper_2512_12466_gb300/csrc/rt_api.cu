@@ -651,16 +651,15 @@ cudaError_t grow_rays(rt_handle* h, int level, int64_t need)
 }
 
 // One march launch: children [c0, c1) of `level`, or as many of them as the device counted (counted).
-// ready: the level's geometry table, if it is in place (null: built here, once per device, or walked).
+// table: the level's geometry table (null: its rays are walked). The next level's ray buffer is in place.
 template <class R>
-int launch_level(rt_handle* h, int level, int64_t c0, int64_t c1, bool counted, bool early, const GeomLevel* ready)
+int launch_level(rt_handle* h, int level, int64_t c0, int64_t c1, bool counted, bool early, const GeomLevel* table)
 {
     char range[32];
     std::snprintf(range, sizeof(range), "march level %d", level);
     NvtxRange nvtx(range);
     // rays of the deepest level end before their split sphere or at level_max
     const bool can_split = level < h->table_level;
-    if (can_split) RT_CUDA(h, grow_rays<R>(h, level + 1, c1 - c0), "ray buffer");
     MarchArgs<R> a;
     a.level = level;
     a.n = h->cfg.n;
@@ -693,22 +692,28 @@ int launch_level(rt_handle* h, int level, int64_t c0, int64_t c1, bool counted, 
     // grid-stride blocks of equal share: 12 per SM is a whole number of waves for the march
     // kernels' 2, 3 and 4 resident blocks per SM, so no last wave runs an SM part-empty
     const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)h->sm_count * kMarchBlocksPerSm));
-    GeomLevel gl;
-    if (ready) gl = *ready;
-    const bool table = ready || (!(h->cfg.flags & RT_FLAG_NO_GEOMETRY_TABLE) &&
-                                 geometry_level(h->device, h->rq, level, h->cfg.n, h->rs, a.dirs, h->stream,
-                                                sizeof(R) == 8, &gl));
     if constexpr (sizeof(R) == 8) {
-        if (table) launch_march_table_f64(a, gl, grid, h->stream);
+        if (table) launch_march_table_f64(a, *table, grid, h->stream);
         else launch_march_f64(a, grid, h->stream);
     } else {
-        if (table) launch_march_table_f32(a, gl, grid, h->stream);
+        if (table) launch_march_table_f32(a, *table, grid, h->stream);
         else launch_march_f32(a, grid, h->stream);
     }
     RT_LAUNCHED(h, "march launch");
     h->launches++;
     h->march_launches++;
     if (table) h->table_levels |= int64_t(1) << level;
+    return RT_OK;
+}
+
+// The time of the launches since the last wait, into ms_march (the stream has been waited for).
+int collect_march(rt_handle* h)
+{
+    if (!h->march_open) return RT_OK;
+    h->march_open = false;
+    float ms = 0.f;
+    RT_CUDA(h, cudaEventElapsedTime(&ms, h->ev[4], h->ev[5]), "event");
+    h->ms_march += ms;
     return RT_OK;
 }
 
@@ -730,31 +735,43 @@ int run_levels(rt_handle* h, int level, int64_t total, bool counted)
         if (level > 0 || c0 > 0)             // the step's first launch finds them cleared
             RT_CUDA(h, cudaMemsetAsync(h->d_count + level + 1, 0,
                                        sizeof(unsigned long long) * (size_t)(RT_MAX_LEVELS - level), h->stream), "counters");
-        int l = level;
-        int64_t bound = c1 - c0;
-        int rc = launch_level<R>(h, l, c0, c1, counted, false, nullptr);
-        if (rc) return rc;
-        while (l < h->table_level && 4 * bound <= kChainChildren) {
-            GeomLevel gl;
+        // ---- the launches that go together: their ray buffers and tables first, outside the timed span
+        const bool tables = !(h->cfg.flags & RT_FLAG_NO_GEOMETRY_TABLE);
+        GeomLevel gl[kMaxLevel + 1];
+        bool table[kMaxLevel + 1];
+        int last = level;
+        if (level < h->table_level) RT_CUDA(h, grow_rays<R>(h, level + 1, c1 - c0), "ray buffer");
+        table[level] = tables && geometry_level(h->device, h->rq, level, h->cfg.n, h->rs,
+                                                h->dirs + healpix_level_offset(level), h->stream, sizeof(R) == 8, &gl[level]);
+        for (int64_t bound = 4 * (c1 - c0); last < h->table_level && bound <= kChainChildren; bound *= 4) {
             GeomState have = GeomState::none;
-            if (!(h->cfg.flags & RT_FLAG_NO_GEOMETRY_TABLE))
-                have = geometry_state(h->device, h->rq, l + 1, h->cfg.n, h->rs, sizeof(R) == 8, &gl);
+            if (tables)
+                have = geometry_state(h->device, h->rq, last + 1, h->cfg.n, h->rs, sizeof(R) == 8, &gl[last + 1]);
             if (have == GeomState::unbuilt) break;
-            if (l + 1 < h->table_level && grow_rays<R>(h, l + 2, 4 * bound) != cudaSuccess) {
+            if (last + 1 < h->table_level && grow_rays<R>(h, last + 2, bound) != cudaSuccess) {
                 cudaGetLastError();          // perhaps enough for the rays there are
                 break;
             }
-            ++l;
-            bound *= 4;
-            rc = launch_level<R>(h, l, 0, bound, true, true, have == GeomState::ready ? &gl : nullptr);
+            table[++last] = have == GeomState::ready;
+        }
+        if (!h->march_open) RT_CUDA(h, cudaEventRecord(h->ev[4], h->stream), "event");
+        h->march_open = true;
+        int64_t bound = c1 - c0;
+        for (int l = level; l <= last; ++l, bound *= 4) {
+            const bool first = l == level;
+            const int rc = launch_level<R>(h, l, first ? c0 : 0, first ? c1 : bound, !first || counted, !first,
+                                           table[l] ? &gl[l] : nullptr);
             if (rc) return rc;
         }
-        if (l == h->table_level) continue;
+        RT_CUDA(h, cudaEventRecord(h->ev[5], h->stream), "event");
+        if (last == h->table_level) continue;
         RT_CUDA(h, cudaMemcpyAsync(h->h_words, h->d_words, sizeof(StepWords), cudaMemcpyDeviceToHost, h->stream), "counter read");
         RT_CUDA(h, cudaStreamSynchronize(h->stream), "march");
         if (h->h_st->bad_input) return RT_OK;                  // nothing was traced; the step ends with the error
         if (h->h_st->err) return fail(h, RT_EDEVICE, "march kernel reported an internal error");
-        rc = run_levels<R>(h, l + 1, 4 * (int64_t)h->h_words->ray_count[l + 1], false);
+        int rc = collect_march(h);
+        if (rc) return rc;
+        rc = run_levels<R>(h, last + 1, 4 * (int64_t)h->h_words->ray_count[last + 1], false);
         if (rc) return rc;
     }
     return RT_OK;
@@ -828,6 +845,8 @@ int trace(rt_handle* h, const double* xuse, bool first)
     h->launches++;
     h->march_launches = 0;
     h->table_levels = 0;
+    h->ms_march = 0.0;
+    h->march_open = false;
     RT_CUDA(h, cudaEventRecord(h->ev[1], h->stream), "event");
     const bool counted = h->n_emit < 0;
     const int64_t total = 12 * (counted ? h->nsrc : h->n_emit);
@@ -1426,7 +1445,6 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
         const int rc = prepare_sources(h);
         if (rc) return rc;
     }
-    h->ms_march = 0.0;
 
     // ---- trace, optionally iterated with the C2-Ray update (Sec. 2.4)
     int iters = 0;
@@ -1450,9 +1468,8 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
             resid = h->h_st->maxdiff;
             if (h->h_st->bad_input) return reject(h);
             if (h->h_st->err) return fail(h, RT_EDEVICE, "march kernel reported an internal error");
-            float ms = 0.f;
-            RT_CUDA(h, cudaEventElapsedTime(&ms, h->ev[1], h->ev[2]), "event");
-            h->ms_march = ms;
+            rc = collect_march(h);
+            if (rc) return rc;
             if (resid < h->cfg.chem_tol || iters >= maxit) break;
             xuse = xnew;
             xnew = xnew == h->d_xavg ? h->d_heat : h->d_xavg;
@@ -1499,6 +1516,8 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
     if (h->h_st->bad_input) return reject(h);
     if (h->h_st->err) return fail(h, RT_EDEVICE, "a kernel reported an internal error");
     finish_sources(h);
+    const int rc_march = collect_march(h);
+    if (rc_march) return rc_march;
 
     if (st) {
         std::memset(st, 0, sizeof(*st));
@@ -1531,7 +1550,7 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
         st->ms_trace = ms;
         cudaEventElapsedTime(&ms, h->ev[0], h->ev[3]);
         st->ms_step = ms;
-        st->ms_march = h->cfg.chem_iterate ? h->ms_march : st->ms_trace;
+        st->ms_march = h->ms_march;
         st->march_launches = h->march_launches;
         for (int l = 0; l < RT_MAX_LEVELS; ++l)                // a level launched in vain read nothing
             if (d.rays[l]) st->table_levels |= h->table_levels & (int64_t(1) << l);

@@ -130,8 +130,9 @@ struct rt_handle {
     nyx::DevStats* h_st = nullptr;           // &h_words->st
     nyx::FieldCheck* h_chk = nullptr;
 
-    cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
+    cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     double ms_march = 0.0;
+    bool march_open = false;         // launches between ev[4] and ev[5] that ms_march does not have yet
     bool fields_set = false;
     bool sticky = false;
     int launches = 0;
