@@ -247,8 +247,10 @@ __global__ void __launch_bounds__(kBlock) prepare_kappa_kernel(const FieldJob J)
 
 __global__ void __launch_bounds__(kBlock) finalize_kernel(const FieldJob J)
 {
-    // nothing goes to the caller's arrays from inputs found invalid or from a trace that reported an error
+    // nothing goes to the caller's arrays from inputs found invalid, from a trace that reported an error or
+    // from one that is not complete
     if (J.valid && (J.st->bad_input || J.st->err)) return;
+    if (J.more && *J.more) return;
     finalize_cells(J, blockIdx.x, gridDim.x);
 }
 
@@ -293,8 +295,10 @@ __global__ void __launch_bounds__(kBlock) chem_kernel(const double* __restrict__
                                                       const double* __restrict__ xavg, double* __restrict__ xnew,
                                                       double* __restrict__ xend,
                                                       const double* __restrict__ gamma, int64_t ncell, double dt,
-                                                      double alpha_B, double C_H, double clump, DevStats* st)
+                                                      double alpha_B, double C_H, double clump,
+                                                      const unsigned long long* more, DevStats* st)
 {
+    if (more && *more) return;
     double md = 0.0;
     for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < ncell; c += (int64_t)gridDim.x * blockDim.x) {
         const double xp = xavg[c];
@@ -365,9 +369,10 @@ int launch_finalize_many(const FieldJob* jobs, const FieldOut* outs, const unsig
 
 int launch_chem_update(const double* nh, const double* x0, const double* xavg, double* xnew, double* xend,
                        const double* gamma, int64_t ncell, double dt, double alpha_B, double C_H, double clump,
-                       DevStats* st, cudaStream_t s)
+                       const unsigned long long* more, DevStats* st, cudaStream_t s)
 {
-    chem_kernel<<<grid_for(ncell), kBlock, 0, s>>>(nh, x0, xavg, xnew, xend, gamma, ncell, dt, alpha_B, C_H, clump, st);
+    chem_kernel<<<grid_for(ncell), kBlock, 0, s>>>(nh, x0, xavg, xnew, xend, gamma, ncell, dt, alpha_B, C_H, clump, more,
+                                                   st);
     return 1;
 }
 

@@ -724,8 +724,11 @@ int collect_march(rt_handle* h)
 // there. So a table is built only for a level that rays reach (levels 0 to 8 of a box of 128^3 cells or
 // more take 0.7 GB in FP32, 1.4 in FP64), and a step fails for want of memory only where its rays need it.
 // counted: `total` is a bound itself (level 0, with the catalog's size on the device).
+// tail: nothing of the trace comes after these levels. Where it then stops before a level without a table
+// it does not wait: most such levels have no rays (the wait cost 10 us a trace of an opaque box), so what
+// follows is enqueued, does nothing if there are some (FieldJob::more), and resume_trace marches them.
 template <class R>
-int run_levels(rt_handle* h, int level, int64_t total, bool counted)
+int run_levels(rt_handle* h, int level, int64_t total, bool counted, bool tail)
 {
     if (total <= 0) return RT_OK;
     if (level > h->table_level || level > kMaxLevel)
@@ -740,14 +743,20 @@ int run_levels(rt_handle* h, int level, int64_t total, bool counted)
         GeomLevel gl[kMaxLevel + 1];
         bool table[kMaxLevel + 1];
         int last = level;
+        bool unbuilt = false;
         if (level < h->table_level) RT_CUDA(h, grow_rays<R>(h, level + 1, c1 - c0), "ray buffer");
-        table[level] = tables && geometry_level(h->device, h->rq, level, h->cfg.n, h->rs,
-                                                h->dirs + healpix_level_offset(level), h->stream, sizeof(R) == 8, &gl[level]);
+        auto state = [&](int l) {            // asks for the budget (a driver call) only where the table is missing
+            return tables ? geometry_state(h->device, h->rq, l, h->cfg.n, h->rs, sizeof(R) == 8, &gl[l]) : GeomState::none;
+        };
+        const GeomState mine = state(level);
+        table[level] = mine == GeomState::ready ||
+                       (mine == GeomState::unbuilt &&
+                        geometry_level(h->device, h->rq, level, h->cfg.n, h->rs, h->dirs + healpix_level_offset(level),
+                                       h->stream, sizeof(R) == 8, &gl[level]));
         for (int64_t bound = 4 * (c1 - c0); last < h->table_level && bound <= kChainChildren; bound *= 4) {
-            GeomState have = GeomState::none;
-            if (tables)
-                have = geometry_state(h->device, h->rq, last + 1, h->cfg.n, h->rs, sizeof(R) == 8, &gl[last + 1]);
-            if (have == GeomState::unbuilt) break;
+            const GeomState have = state(last + 1);
+            unbuilt = have == GeomState::unbuilt;
+            if (unbuilt) break;
             if (last + 1 < h->table_level && grow_rays<R>(h, last + 2, bound) != cudaSuccess) {
                 cudaGetLastError();          // perhaps enough for the rays there are
                 break;
@@ -765,15 +774,43 @@ int run_levels(rt_handle* h, int level, int64_t total, bool counted)
         }
         RT_CUDA(h, cudaEventRecord(h->ev[5], h->stream), "event");
         if (last == h->table_level) continue;
+        const bool tail_slice = tail && c1 == total;
+        if (unbuilt && tail_slice) {
+            h->pending_level = last + 1;
+            return RT_OK;
+        }
         RT_CUDA(h, cudaMemcpyAsync(h->h_words, h->d_words, sizeof(StepWords), cudaMemcpyDeviceToHost, h->stream), "counter read");
         RT_CUDA(h, cudaStreamSynchronize(h->stream), "march");
         if (h->h_st->bad_input) return RT_OK;                  // nothing was traced; the step ends with the error
         if (h->h_st->err) return fail(h, RT_EDEVICE, "march kernel reported an internal error");
         int rc = collect_march(h);
         if (rc) return rc;
-        rc = run_levels<R>(h, last + 1, 4 * (int64_t)h->h_words->ray_count[last + 1], false);
+        rc = run_levels<R>(h, last + 1, 4 * (int64_t)h->h_words->ray_count[last + 1], false, tail_slice);
         if (rc) return rc;
     }
+    return RT_OK;
+}
+
+// The count of rays that the last trace may have left to resume_trace (null: none).
+const unsigned long long* rays_left(const rt_handle* h)
+{
+    return h->pending_level > 0 ? h->d_count + h->pending_level : nullptr;
+}
+
+// After a wait, with h_words read: the rays that the last trace left, if any (*resumed), marched to the end.
+int resume_trace(rt_handle* h, bool* resumed)
+{
+    const int level = h->pending_level;
+    h->pending_level = 0;
+    *resumed = level > 0 && h->h_words->ray_count[level] > 0;
+    if (!*resumed) return RT_OK;
+    int rc = collect_march(h);
+    if (rc) return rc;
+    const int64_t total = 4 * (int64_t)h->h_words->ray_count[level];
+    rc = h->cfg.precision == RT_FP32 ? run_levels<float>(h, level, total, false, true)
+                                     : run_levels<double>(h, level, total, false, true);
+    if (rc) return rc;
+    RT_CUDA(h, cudaEventRecord(h->ev[2], h->stream), "event");
     return RT_OK;
 }
 
@@ -847,11 +884,12 @@ int trace(rt_handle* h, const double* xuse, bool first)
     h->table_levels = 0;
     h->ms_march = 0.0;
     h->march_open = false;
+    h->pending_level = 0;
     RT_CUDA(h, cudaEventRecord(h->ev[1], h->stream), "event");
     const bool counted = h->n_emit < 0;
     const int64_t total = 12 * (counted ? h->nsrc : h->n_emit);
-    const int rc = h->cfg.precision == RT_FP32 ? run_levels<float>(h, 0, total, counted)
-                                               : run_levels<double>(h, 0, total, counted);
+    const int rc = h->cfg.precision == RT_FP32 ? run_levels<float>(h, 0, total, counted, true)
+                                               : run_levels<double>(h, 0, total, counted, true);
     if (rc) return rc;
     RT_CUDA(h, cudaEventRecord(h->ev[2], h->stream), "event");
     return RT_OK;
@@ -1459,15 +1497,19 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
             int rc = trace(h, xuse, iters == 0);
             if (rc) return rc;
             ++iters;
-            h->launches += launch_chem_update(h->d_nh, h->d_x, xuse, xnew, h->d_xend, h->d_gamma, h->ncell, dt_s,
-                                              h->cfg.alpha_B, h->cfg.C_H, h->cfg.clumping, h->d_st, s);
-            RT_LAUNCHED(h, "chemistry launch");
-            // the residual, and the error words
-            RT_CUDA(h, cudaMemcpyAsync(h->h_words, h->d_words, sizeof(StepWords), cudaMemcpyDeviceToHost, s), "residual read");
-            RT_CUDA(h, cudaStreamSynchronize(s), "chemistry");
+            for (bool again = true; again;) {
+                h->launches += launch_chem_update(h->d_nh, h->d_x, xuse, xnew, h->d_xend, h->d_gamma, h->ncell, dt_s,
+                                                  h->cfg.alpha_B, h->cfg.C_H, h->cfg.clumping, rays_left(h), h->d_st, s);
+                RT_LAUNCHED(h, "chemistry launch");
+                // the residual, the error words and the rays left
+                RT_CUDA(h, cudaMemcpyAsync(h->h_words, h->d_words, sizeof(StepWords), cudaMemcpyDeviceToHost, s), "residual read");
+                RT_CUDA(h, cudaStreamSynchronize(s), "chemistry");
+                if (h->h_st->bad_input) return reject(h);
+                if (h->h_st->err) return fail(h, RT_EDEVICE, "march kernel reported an internal error");
+                rc = resume_trace(h, &again);
+                if (rc) return rc;
+            }
             resid = h->h_st->maxdiff;
-            if (h->h_st->bad_input) return reject(h);
-            if (h->h_st->err) return fail(h, RT_EDEVICE, "march kernel reported an internal error");
             rc = collect_march(h);
             if (rc) return rc;
             if (resid < h->cfg.chem_tol || iters >= maxit) break;
@@ -1494,27 +1536,31 @@ int rt_step(rt_handle* h, double dt_s, double* gamma_out, double* heat_out, int 
     job.valid = h->d_chk;
     job.gamma_out = gamma_direct ? gamma_out : nullptr;
     job.heat = heat_direct ? heat_out : (heat_out ? h->d_heat : nullptr);
-    h->launches += launch_finalize(job, s);
-    RT_LAUNCHED(h, "finalize launch");
-    if (h->cfg.chem_iterate) {
-        RT_CUDA(h, cudaMemcpyAsync(h->d_x, h->d_xend, fb, cudaMemcpyDeviceToDevice, s), "x update");   // x(t + dt)
-        h->fields_checked = false;
-    }
-    const cudaMemcpyKind k = where == RT_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
-    if ((gamma_out && !gamma_direct) || (heat_out && !heat_direct)) {
-        // nothing is copied over the caller's data before the inputs and the trace are known to be sound
-        RT_CUDA(h, cudaMemcpyAsync(h->h_words, h->d_words, sizeof(StepWords), cudaMemcpyDeviceToHost, s), "input check");
+    const bool copies = (gamma_out && !gamma_direct) || (heat_out && !heat_direct);
+    for (bool again = true; again;) {
+        job.more = rays_left(h);
+        h->launches += launch_finalize(job, s);
+        RT_LAUNCHED(h, "finalize launch");
+        if (h->cfg.chem_iterate) {
+            RT_CUDA(h, cudaMemcpyAsync(h->d_x, h->d_xend, fb, cudaMemcpyDeviceToDevice, s), "x update");   // x(t + dt)
+            h->fields_checked = false;
+        }
+        if (!copies) RT_CUDA(h, cudaEventRecord(h->ev[3], s), "event");
+        RT_CUDA(h, cudaMemcpyAsync(h->h_words, h->d_words, sizeof(StepWords), cudaMemcpyDeviceToHost, s), "stats read");
         RT_CUDA(h, cudaStreamSynchronize(s), "step");
+        // nothing goes to the caller before the inputs and the trace are known to be sound
         if (h->h_st->bad_input) return reject(h);
         if (h->h_st->err) return fail(h, RT_EDEVICE, "a kernel reported an internal error");
+        const int rc = resume_trace(h, &again);
+        if (rc) return rc;
     }
-    if (gamma_out && !gamma_direct) RT_CUDA(h, cudaMemcpyAsync(gamma_out, h->d_gamma, fb, k, s), "gamma copy");
-    if (heat_out && !heat_direct) RT_CUDA(h, cudaMemcpyAsync(heat_out, h->d_heat, fb, k, s), "heat copy");
-    RT_CUDA(h, cudaEventRecord(h->ev[3], s), "event");
-    RT_CUDA(h, cudaMemcpyAsync(h->h_words, h->d_words, sizeof(StepWords), cudaMemcpyDeviceToHost, s), "stats read");
-    RT_CUDA(h, cudaStreamSynchronize(s), "step");
-    if (h->h_st->bad_input) return reject(h);
-    if (h->h_st->err) return fail(h, RT_EDEVICE, "a kernel reported an internal error");
+    if (copies) {
+        const cudaMemcpyKind k = where == RT_HOST ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
+        if (gamma_out && !gamma_direct) RT_CUDA(h, cudaMemcpyAsync(gamma_out, h->d_gamma, fb, k, s), "gamma copy");
+        if (heat_out && !heat_direct) RT_CUDA(h, cudaMemcpyAsync(heat_out, h->d_heat, fb, k, s), "heat copy");
+        RT_CUDA(h, cudaEventRecord(h->ev[3], s), "event");
+        RT_CUDA(h, cudaStreamSynchronize(s), "step");
+    }
     finish_sources(h);
     const int rc_march = collect_march(h);
     if (rc_march) return rc_march;

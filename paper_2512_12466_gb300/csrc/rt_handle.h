@@ -132,6 +132,7 @@ struct rt_handle {
 
     cudaEvent_t ev[6] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
     double ms_march = 0.0;
+    int pending_level = 0;           // level whose rays, if there are any, the last trace has left (0: none)
     bool march_open = false;         // launches between ev[4] and ev[5] that ms_march does not have yet
     bool fields_set = false;
     bool sticky = false;

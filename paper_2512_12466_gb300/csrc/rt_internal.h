@@ -81,6 +81,8 @@ struct FieldJob {
     const FieldCheck* chk = nullptr; // given: n_th from there
     const FieldCheck* valid = nullptr; // given: its invalid cells go to st->bad_input before the trace, and
                                        // where that or st->err is not zero no result is written
+    const unsigned long long* more = nullptr;  // given: rays still to be marched; while there are any no result
+                                               // is written
     DevStats* st = nullptr;
     uint32_t block0 = 0;
 };
@@ -227,9 +229,10 @@ int launch_prepare_many(const FieldJob* jobs, int njobs, uint32_t blocks, bool f
 // outs[i] replaces jobs[i].gamma_out and heat; nothing is written where *err is set.
 int launch_finalize_many(const FieldJob* jobs, const FieldOut* outs, const unsigned* err, int njobs, uint32_t blocks,
                          cudaStream_t s);
+// more as in FieldJob: nothing is done while there are rays to march.
 int launch_chem_update(const double* nh, const double* x0, const double* xavg, double* xnew, double* xend,
                        const double* gamma, int64_t ncell, double dt, double alpha_B, double C_H, double clump,
-                       DevStats* st, cudaStream_t s);
+                       const unsigned long long* more, DevStats* st, cudaStream_t s);
 
 // Small device-to-host readbacks (statistics, counters), written by one kernel straight into mapped
 // pinned host memory: unlike copies they do not queue on the copy engines behind large transfers

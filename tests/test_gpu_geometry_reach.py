@@ -67,3 +67,28 @@ def test_tables_follow_the_rays(precision):
         ref = oracle.run_workload(w, precision=precision, n_th_cm3=0.3 * float(w.n_h.mean()))["stats"]
         for k in ("rays", "segments", "secondary", "dropped_tau"):
             assert list(st[k]) == list(ref[k]), k
+
+
+@pytest.mark.parametrize("where", ["host", "device"])
+def test_chemistry_on_a_grid_without_tables(where):
+    # the update and the results enqueued behind a trace that stops before an unbuilt level wait for its rays
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_2512_12466_gb300 as nyx
+    w = I.stromgren_test("A", 32)
+    kw = {k: w.params[k] for k in ("tau_max", "chem_iterate", "alpha_B", "clumping", "C_H")}
+    kw.update(n_th_cm3=1e-5, n_min_ray=4.3 if where == "host" else 4.4)
+    dt = 10.0 * I.MYR_S
+    ref = oracle.run(w.n_h, w.x_ion, w.cells, w.ndot, w.box_cm, dt_s=dt, **kw)
+    out = torch.full((2, w.n ** 3), np.nan, dtype=torch.float64, device="cuda")
+    for _ in range(2):                                      # without tables, then with
+        s = nyx.Solver(w.n, w.box_cm, **kw)
+        s.set_fields(w.n_h.ravel(), w.x_ion.ravel())
+        s.add_sources(w.cells.ravel(), w.ndot)
+        gamma, heat, st = s.step(dt) if where == "host" else s.step(dt, out[0], out[1])
+        gamma, heat, x = [np.asarray(a.cpu() if hasattr(a, "cpu") else a).ravel() for a in (gamma, heat, s.get_x())]
+        s.close()
+        assert sum(1 for r in st["rays"] if r) > 4
+        assert abs(st["chem_iters"] - ref["stats"]["chem_iters"]) <= 1
+        for got, want in ((gamma, ref["gamma"]), (heat, ref["heat"]), (x, ref["x"])):
+            assert np.linalg.norm(got - want.ravel()) / np.linalg.norm(want) < 1e-8
