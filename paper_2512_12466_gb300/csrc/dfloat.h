@@ -104,6 +104,21 @@ __device__ __forceinline__ dflt df_of(const double x)
     return {h, l};
 }
 
+// df_of with the head rounded to nearest, so that the tail is at most half a unit of it and keeps one bit
+// more (an error of 2^-49 of the value instead of 2^-48).
+__device__ __forceinline__ dflt df_of_near(const double x)
+{
+    const long long b = __double_as_longlong(x);
+    const unsigned hw = (unsigned)(b >> 32), lw = (unsigned)b;
+    const int e = (int)(hw >> 20);
+    if (e < 897) return {0.f, 0.f};
+    const unsigned up = (lw >> 28) & 1u;                     // the tail's leading bit
+    const float h = __uint_as_float((((unsigned)(e - 896) << 23) | ((hw & 0xfffffu) << 3) | (lw >> 29)) + up);
+    const int tail = (int)(lw & 0x1fffffffu) - (int)(up << 29);
+    const float l = e >= 949 ? __fmul_rn(__int2float_rn(tail), __uint_as_float((unsigned)(e - 948) << 23)) : 0.f;
+    return {h, l};
+}
+
 // df_of for a positive double in [2^-74, 2^127), without the range tests (segment lengths: the
 // integer traversal makes every segment longer than about 2^-46 cells)
 __device__ __forceinline__ dflt df_of_len(const double x)

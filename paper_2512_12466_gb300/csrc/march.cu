@@ -25,6 +25,7 @@
 
 #include "rt_internal.h"
 #include "dfloat.h"
+#include "exp_table.h"
 #include "rate_table.h"
 
 namespace nyx {
@@ -1192,7 +1193,7 @@ __device__ __forceinline__ bool march_ray_table(const SolveView<R>& V, const Geo
 //   - the Eqs. 5-8 shares and the Eq. 8 ratio kap / kap' (a reciprocal and one correction).
 // Each deposit is rounded to double by integer operations (df_to_double_pos) for its atomic add.
 // From dtau = 2 on (an opaque cell, where most of the budget goes at once) the deposits are FP64, with
-// e^{-dtau} from the same rate table (exp_minus) and quotients from double-float reciprocals (quot_pos).
+// e^{-dtau} from tables (exp_minus) and quotients from double-float reciprocals (quot_pos).
 
 // The rate table in shared memory: two float4 arrays, row j's {c0, c0', c1, c1'} at 4 j and its
 // {c2, c2', c3, c4} at 4 (kRateIntervals + j), so each is one 16-byte load.
@@ -1233,7 +1234,7 @@ __device__ __forceinline__ dflt rate_factor(const float* __restrict__ tab, const
 }
 
 // e^{-2 m} for m = 0 .. 27 as double-floats (from the exponential series in 40-digit arithmetic); from
-// m = 27 on e^{-x} is below 2^-76, nothing beside 1.
+// m = 28 on e^{-x} is below 2^-79, nothing beside 1.
 constexpr int kExpRows = 28;
 __device__ constexpr float2 kExpMinus2[kExpRows] = {
     {1.0e+00f, 0.0e+00f}, {1.3533528e-01f, 1.7453331e-09f},
@@ -1252,17 +1253,30 @@ __device__ constexpr float2 kExpMinus2[kExpRows] = {
     {2.610279e-23f, 2.3214166e-31f}, {3.5326284e-24f, 1.8138574e-31f},
 };
 
-// e^{-x} for a segment of optical depth x >= 2 (a double-float), from the rate table: with x = 2 m + r,
-// 0 <= r < 2, it is e^{-2 m} (1 - r g(r)). Its error, about 2^-46 of itself, is below 2^-48 of 1 - e^{-x}.
-__device__ __forceinline__ dflt exp_minus(const float* __restrict__ tab, const dflt x)
+// e^{-x} for the optical depth 2 <= x < 64 of an opaque segment, to 3 2^-53 of itself (and the error of its
+// row of kExpMinus2, 2^-49 at worst, 2^-53 below x = 4): x is split exactly, as an integer of units 2^-51,
+// into 2 m + j / 256 + r with |r| <= 1/512, and e^{-r} - 1 summed as a double-float (2^-54 of 1), with the
+// rest of the middle factor in its tail. Four FP64 operations; a double-float product with the rate table
+// took one, but kept only 2^-44 of what the segment leaves of the budget.
+__device__ __forceinline__ double exp_minus(const double x)
 {
-    const int m = (int)fminf(0.5f * x.h, (float)(kExpRows - 1));
-    if (m >= kExpRows - 1) return {0.f, 0.f};
-    const dflt r = df_fast_two_sum(__fsub_rn(x.h, (float)(2 * m)), x.l);      // the head difference is exact
-    const dflt u = df_mul(r, rate_factor(tab, r));
-    const dflt e = df_add(dflt{1.f, 0.f}, dflt{-u.h, -u.l});
-    const float2 c = kExpMinus2[m];
-    return df_mul(e, dflt{c.x, c.y});
+    const long long b = __double_as_longlong(x);
+    const unsigned long long units =
+        ((((unsigned long long)b & 0xfffffffffffffull) | 0x10000000000000ull) << ((int)(b >> 52) - 1024)) + (1ull << 42);
+    const int m = (int)(units >> 52), j = (int)(units >> 43) & 511;
+    if (m >= kExpRows) return 0.0;
+    const long long rem = (long long)(units & ((1ull << 43) - 1)) - (1ll << 42);
+    // r = rh + rl, exactly
+    const dflt r = df_fast_two_sum(__fmul_rn(__int2float_rn((int)(rem >> 19)), 2.3283064365386963e-10f),        // 2^-32
+                                   __fmul_rn(__int2float_rn((int)(rem & 0x7ffff)), 4.440892098500626e-16f));   // 2^-51
+    // e^{-r} - 1 = r^2 (1/2 - r / 6 + r^2 / 24 - r^3 / 120) - r
+    const float c = __fmul_rn(r.h, __fmaf_rn(r.h, __fmaf_rn(r.h, -1.0f / 120.0f, 1.0f / 24.0f), -1.0f / 6.0f));
+    dflt p = df_add(df_mul(df_mul(r, r), dflt{0.5f, c}), dflt{-r.h, -r.l});
+    p.l = __fadd_rn(p.l, kExpFracRest[j]);
+    const double f = kExpFrac[j];
+    const double e = __fma_rn(f, df_to_double(p, 0), f);
+    const float2 t = kExpMinus2[m];
+    return __fma_rn(e, widen_scaled(t.x, 0), __dmul_rn(e, widen_scaled(t.y, 0)));
 }
 
 // a / b for positive normal doubles, to about an ulp: the reciprocal of b's mantissa as a double-float
@@ -1380,18 +1394,16 @@ struct OpaqueSeg {
     double aQ, wd;
     dflt Q;
 };
-__device__ __noinline__ OpaqueSeg opaque_segment(const float* __restrict__ rtab, const dflt Q, const double dtau,
-                                                 const double kap)
+__device__ __noinline__ OpaqueSeg opaque_segment(const dflt Q, const double dtau, const double kap)
 {
     // in FP64, where most of the budget goes at once, but without the exponential and the division of
-    // that unit: some fifteen operations (64 cycles of its pipe each) instead of about sixty. The
-    // 64^3 Stromgren step (neutral gas, Delta tau up to 3.5): 4.33 -> 3.63 ms.
-    const double ed = Ieee<double>::lt(dtau, 64.0) ? df_to_double(exp_minus(rtab, df_of(dtau)), 0) : 0.0;
+    // that unit: some twenty operations (64 cycles of its pipe each) instead of about sixty
+    const double ed = Ieee<double>::lt(dtau, 64.0) ? exp_minus(dtau) : 0.0;
     const double Qd = df_to_double(Q, 0);
     OpaqueSeg o;
     o.aQ = Qd * (1.0 - ed);
     o.wd = quot_pos(o.aQ, kap);
-    o.Q = df_of(Qd * ed);
+    o.Q = df_of_near(Qd * ed);
     return o;
 }
 
@@ -1536,7 +1548,7 @@ __device__ __forceinline__ bool march_ray_table_df(const SolveView<double>& V, c
                 w = df_mul(Q, dsf);                       // optically thin limit
             }
         } else {
-            const OpaqueSeg o = opaque_segment(rtab, Q, dtau, kap);
+            const OpaqueSeg o = opaque_segment(Q, dtau, kap);
             aQ = o.aQ;
             wd = o.wd;
             Q = o.Q;
