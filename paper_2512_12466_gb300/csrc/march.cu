@@ -1397,7 +1397,9 @@ struct OpaqueSeg {
 __device__ __noinline__ OpaqueSeg opaque_segment(const dflt Q, const double dtau, const double kap)
 {
     // in FP64, where most of the budget goes at once, but without the exponential and the division of
-    // that unit: some twenty operations (64 cycles of its pipe each) instead of about sixty
+    // that unit: some twenty operations (64 cycles of its pipe each) instead of about sixty. The 64^3
+    // Stromgren step (neutral gas, dtau up to 3.5): 3.56 ms, with expm1 and the divisions 3.98; the
+    // half-ionized 165^3 box: 0.418 and 0.456.
     const double ed = Ieee<double>::lt(dtau, 64.0) ? exp_minus(dtau) : 0.0;
     const double Qd = df_to_double(Q, 0);
     OpaqueSeg o;

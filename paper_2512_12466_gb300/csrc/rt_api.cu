@@ -42,8 +42,8 @@ constexpr int64_t kMaxChildrenPerLaunch = int64_t(1) << 27;
 // Levels that can hold at most this many rays are launched one behind the other without the host
 // knowing their size: each launch takes it from the count the level before it left on the device. The
 // bound is what the next level's ray buffer is sized for (24 bytes a record, 50 MB). A host round trip
-// costs 15-25 us, which for a level of a million rays is below a tenth of its march; four levels launched
-// in vain (an opaque box whose rays end at level 0) cost 2.5 us each.
+// costs 15-25 us, which for a level of a million rays is below a tenth of its march; a level launched in
+// vain (an opaque box whose rays end earlier) costs 2.5 us.
 constexpr int64_t kChainChildren = int64_t(1) << 21;
 constexpr int kMarchBlock = 256;
 constexpr int kMarchBlocksPerSm = 12;

@@ -9,7 +9,7 @@
 // The stage is bound by launches and by serial chains, not by bytes (32768
 // sources are 0.7 MB): a catalog of up to kSmallSources is one launch of one
 // block, a larger one a tiled radix sort (one block for all of it took 134 us
-// at 32768 keys) and prefix sums folded into the kernels that need them. Sizes
+// at 32768 keys, the tiles take 33) and prefix sums folded into the kernels that need them. Sizes
 // that the device counts (after dedup, of the positive radii, of the groups)
 // stay there. The FP64 pipe (64 cycles a warp instruction) is kept for results.
 #include <algorithm>
@@ -112,6 +112,8 @@ __device__ __forceinline__ double warp_sum(double v)
 // The whole stage for up to kSmallSources sources in one block: validation, the stable sort by cell
 // (bitonic on (cell key, index), which is unique), the sums over equal cells in index order, and the
 // emitted catalog (emit null: only cells and rates). Ten launches and their gaps otherwise.
+// The line at 2048 (16 KB of keys): the block's time grows with the catalog (a 64^3 opaque step takes 133 us
+// with 1024 sources, 143 with 2048), the tiles' hardly (162 with 2049, 174 with 4096), so beyond it the two meet.
 constexpr int kSmallSources = 2048;
 
 __global__ void __launch_bounds__(1024) small_sources_kernel(const int32_t* __restrict__ cells,
@@ -210,7 +212,7 @@ __global__ void cell_keys_kernel(const int32_t* __restrict__ cells, const double
 // (a warp owns a contiguous chunk of it), two launches a pass. The first counts every tile's digits; the
 // second takes each tile's base for a digit from the counts (all smaller digits, and the same digit in
 // the tiles before), then each warp places its chunk in sequence order, 32 keys an iteration, a lane after
-// the lower lanes that share its digit (8 ballots). 32768 keys of 24 bits: 134 -> 45 us.
+// the lower lanes that share its digit (8 ballots). 32768 keys of 24 bits: 33 us, one block for all 134.
 constexpr int kSortTile = 1024;
 constexpr int kSortBlocks = 512;
 constexpr int kSortWarps = kBlock / 32;
@@ -446,8 +448,8 @@ __global__ void __launch_bounds__(kBlock) radius_kernel(const int32_t* __restric
 // cell is c plus floor(1/2 + r d), the same offset for every source. So the distinct offsets of each shell
 // are found once (shell_kernel, a block a shell) and a source only looks its cells up, a warp each. With
 // periodic boundaries the grid has to be wider than the largest shell, so that no two offsets meet.
-// 29815 sources of a 256^3 box: 376 us (radius_kernel: a sort of every shell of
-// every source) -> 67.
+// 29815 sources of a 256^3 box: 72 us (13 for the tables), against 376 with radius_kernel (a sort of every
+// shell of every source).
 constexpr int kMaxShells = 128;
 constexpr int kShellBias = 512;
 
@@ -612,8 +614,8 @@ __global__ void __launch_bounds__(kBlock) compact_kernel(const int32_t* __restri
 // larger root is hooked under the smaller, so each component's root is its smallest index. A block takes
 // a tile of kBlock x kPairTile pairs: a thread one source against the tile's others, in shared memory.
 // Almost all pairs are far apart, which integer and float arithmetic settles (the float limit is above
-// the FP64 one by more than its rounding); the others take the exact test. 161 -> 98 us for the
-// ionized sources among 29815.
+// the FP64 one by more than its rounding); the others take the exact test. 88 us for the ionized
+// sources among 29815; 161 with the exact test for every pair.
 constexpr int kPairTile = 256;
 
 // minimg of an offset between two cells of the grid, |d| < n
