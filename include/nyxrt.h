@@ -146,8 +146,8 @@ typedef struct rt_stats {
     double ms_step;            /* device time of the whole step */
     double ms_march;           /* device time of the last trace's march launches: the sum over the runs of
                                   launches that follow one another without the host, each from its
-                                  first launch to the end of its last (CUDA events); host waits, table
-                                  builds and the growth of ray buffers are not in it */
+                                  first launch to the end of its last (CUDA events); host waits and
+                                  table builds are not in it */
     int64_t march_launches;    /* march kernel launches in the last trace */
     int64_t table_levels;      /* bit l set: level l's march read its cells from the per-device
                                   geometry tables in the last trace; clear: it walked its rays

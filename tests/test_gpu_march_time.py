@@ -1,4 +1,4 @@
-"""rt_stats.ms_march is the time of the march launches, without the table builds, buffer growth and host waits that a
+"""rt_stats.ms_march is the time of the march launches, without the table builds and host waits that a
 grid's first step has between them: the first step of a grid size reports about what the second does, far less
 than its whole trace. (A build of this grid's FP64 tables takes tens of milliseconds, its march about one.)"""
 import pytest
