@@ -48,10 +48,10 @@ L2_FLUSH_BYTES = 512 << 20
 # [--precision fp64]`), scaled to the full workload by primary segments. Valid only for the kernel
 # sources it was taken on.
 TRAFFIC_CAPTURE = {"kernel": "march_table_kernel",
-                   "bytes_per_segment": {"fp32": 8.626376059933783, "fp64": 19.1181517084529},
-                   "sources": {"paper_2512_12466_gb300/csrc/march.cu": "17d4ef3d9baa504b",
-                               "paper_2512_12466_gb300/csrc/rt_internal.h": "d0567305ea6de2d9",
-                               "paper_2512_12466_gb300/csrc/dfloat.h": "459135c9d92ee117"}}
+                   "bytes_per_segment": {"fp32": 8.611169955877317, "fp64": 19.12124542586409},
+                   "sources": {"paper_2512_12466_gb300/csrc/march.cu": "26cad099e6d9e756",
+                               "paper_2512_12466_gb300/csrc/rt_internal.h": "c6d0f5f9aab722da",
+                               "paper_2512_12466_gb300/csrc/dfloat.h": "66bb33bd0a50d72d"}}
 
 
 def traffic_per_launch(segments_per_step: float, launches_per_step: float, precision: str = "fp32"):
@@ -803,7 +803,7 @@ def run_nyx(args, world, rank, local):
                               / max(1, f64["march_launches_per_step"]),
                               "kernel": "march_table_kernel<double> (FP64, geometry tables, double-float)",
                               "bound": "instruction issue of the double-float arithmetic (ncu, one level-7 launch: "
-                                       "issue 68% active, 322 thread instructions per segment at 25.3 of 32 lanes, "
+                                       "issue 70% active, 317 thread instructions per segment at 25.1 of 32 lanes, "
                                        "FP64 pipe 31%, DRAM 9%, before the neighbour cell became selects)"}},
         "e2e": {"value": e2e_val, "unit": "segments/s", "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,
                 "steps": e2e_steps},
