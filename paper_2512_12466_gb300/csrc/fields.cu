@@ -13,9 +13,10 @@
 // deposited photons and the results' way out.
 // At 128^3 cells (neutral, FP32) the check takes 16 us, kappa 17 and the heating 14; at 256^3 (half
 // ionized) 82, 102 and 176. Before, kappa took 31 and 220 and the heating 35 and 203, beside a validation, a
-// mean, the clearing of Gamma and two copies each way. A batch of 48 solves takes 231 and 128 us for kappa and
+// mean, the clearing of Gamma and two copies each way. A batch of 48 solves takes 226 and 127 us for kappa and
 // heating, one launch each; 48 launches of each took 13 and 18 us apiece.
 #include <algorithm>
+#include <cmath>
 #include <cstdint>
 
 #include "rt_internal.h"
@@ -121,39 +122,40 @@ __global__ void __launch_bounds__(kBlock) check_fields_kernel(const double* __re
     }
 }
 
-// v rounded to the nearest float, ties to even, on the integer pipe: the magnitude's leading 24 bits and
-// the rest, shifted down first where the result is subnormal; the sign is carried over.
-__device__ __forceinline__ float narrow(const double v)
+// v rounded to the nearest float, ties to even, on the integer pipe, its sign bit changed by flip (0 or
+// 0x80000000): the magnitude's leading 24 bits and the rest, shifted down first where the result is
+// subnormal. Negative values pass through the branch of the values that are no normal floats, so that they
+// cost the others nothing (both shifts drop the sign bit).
+__device__ __forceinline__ float narrow(const double v, unsigned flip)
 {
-    const unsigned sign = (unsigned)(bits_of(v) >> 32) & 0x80000000u;
-    const unsigned hi = (unsigned)(bits_of(v) >> 32) & 0x7fffffffu, lo = (unsigned)bits_of(v);
+    const unsigned hi = (unsigned)(bits_of(v) >> 32), lo = (unsigned)bits_of(v);
     unsigned u = ((hi - 0x38000000u) << 3) | (lo >> 29), rem = lo << 3;       // rem: in units of 2^-32 of u's last place
-    if (hi - 0x38100000u >= 0x47f00000u - 0x38100000u) {                      // not a normal float (zero among them)
-        if (hi >= 0x47f00000u)
-            return __uint_as_float(sign | (hi > 0x7ff00000u || (hi == 0x7ff00000u && lo) ? 0x7fffffffu : 0x7f800000u));
-        const int down = 897 - (int)(hi >> 20);                               // 1 .. 897
-        const unsigned long long m = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
-        const unsigned long long w = down < 32 ? m >> down : 0ull;            // below 2^-158: nothing
-        const bool sticky = down < 32 && (m & ((1ull << down) - 1ull)) != 0ull;
-        u = (unsigned)(w >> 29);
-        rem = ((unsigned)w << 3) | (sticky ? 1u : 0u);
+    if (hi - 0x38100000u >= 0x47f00000u - 0x38100000u) {                      // negative, or not a normal float (zero among them)
+        const unsigned mag = hi & 0x7fffffffu;
+        flip ^= hi & 0x80000000u;
+        if (mag >= 0x47f00000u)
+            return __uint_as_float(flip ^ (mag > 0x7ff00000u || (mag == 0x7ff00000u && lo) ? 0x7fffffffu : 0x7f800000u));
+        if (mag < 0x38100000u) {
+            const int down = 897 - (int)(mag >> 20);                          // 1 .. 897
+            const unsigned long long m = ((unsigned long long)((mag & 0xfffffu) | 0x100000u) << 32) | lo;
+            const unsigned long long w = down < 32 ? m >> down : 0ull;        // below 2^-158: nothing
+            const bool sticky = down < 32 && (m & ((1ull << down) - 1ull)) != 0ull;
+            u = (unsigned)(w >> 29);
+            rem = ((unsigned)w << 3) | (sticky ? 1u : 0u);
+        }
     }
     u += (rem > 0x80000000u || (rem == 0x80000000u && (u & 1u))) ? 1u : 0u;
-    return __uint_as_float(sign | u);
+    return __uint_as_float(u ^ flip);
 }
 
-// n_th's place in the order of bit patterns; above every density where it is a NaN of either sign (no cell
-// is eligible then, as none compares >= to it).
-__device__ __forceinline__ long long threshold_bits(const double n_th)
-{
-    const long long b = bits_of(n_th);
-    return (b & 0x7fffffffffffffffll) > 0x7ff0000000000000ll ? 0x7fffffffffffffffll : b;
-}
+// n_th for eligible: a NaN of either sign as the positive one, whose bit pattern lies above every density's
+// (no cell is eligible then, as none compares >= to it).
+inline double ordered_threshold(const double n_th) { return std::isnan(n_th) ? std::fabs(n_th) : n_th; }
 
-// Eqs. 7-8: whether a cell may receive a secondary deposit, n_H >= n_th and n_HI > 0.
-__device__ __forceinline__ bool eligible(const double nh, const double nhi, const long long th)
+// Eqs. 7-8: whether a cell may receive a secondary deposit, n_H >= n_th and n_HI > 0, on the bit patterns.
+__device__ __forceinline__ bool eligible(const double nh, const double nhi, const double n_th)
 {
-    return bits_of(nh) >= th && bits_of(nhi) > 0;
+    return bits_of(nh) >= bits_of(n_th) && bits_of(nhi) > 0;
 }
 
 // k where the cell may receive a secondary deposit, -k elsewhere, for any sign of k (a -0.0 in n_H gives a
@@ -161,7 +163,7 @@ __device__ __forceinline__ bool eligible(const double nh, const double nhi, cons
 template <class R>
 __device__ __forceinline__ R stored_kappa(const double k, const bool elig)
 {
-    if constexpr (sizeof(R) == 4) return __uint_as_float(__float_as_uint(narrow(k)) ^ (elig ? 0u : 0x80000000u));
+    if constexpr (sizeof(R) == 4) return narrow(k, elig ? 0u : 0x80000000u);
     else return __longlong_as_double(bits_of(k) ^ (elig ? 0ll : (long long)0x8000000000000000ull));
 }
 
@@ -173,7 +175,7 @@ __device__ __forceinline__ R stored_kappa(const double k, const bool elig)
 template <class R>
 __device__ __forceinline__ void prepare_cells(const FieldJob& J, const int64_t first, const int64_t stride)
 {
-    const long long th = threshold_bits(J.chk ? J.chk->n_th : J.n_th);
+    const double n_th = J.chk ? J.chk->n_th : J.n_th;
     R* const kap = static_cast<R*>(J.kap);
     for (int64_t t0 = first * kTile; t0 < J.ncell; t0 += stride * kTile) {
         double a[kUnroll], b[kUnroll];
@@ -189,7 +191,7 @@ __device__ __forceinline__ void prepare_cells(const FieldJob& J, const int64_t f
             if (c >= J.ncell) break;
             const double nhi = __dmul_rn(__dsub_rn(1.0, b[u]), a[u]);
             const double k = __dmul_rn(J.sdx, nhi);
-            kap[c] = stored_kappa<R>(k, eligible(a[u], nhi, th));
+            kap[c] = stored_kappa<R>(k, eligible(a[u], nhi, n_th));
             J.gamma[c] = 0.0;
         }
     }
@@ -280,11 +282,12 @@ __global__ void __launch_bounds__(kBlock) finalize_many_kernel(const FieldJob* _
                                                                const FieldOut* __restrict__ outs,
                                                                const unsigned* err, int njobs)
 {
-    if (*err) return;                             // of any solve: the run fails and no result is written
+    const unsigned failed = *err;                 // of any solve; requested with the search for the job
     const int j = job_of_block(jobs, njobs);
     FieldJob J = jobs[j];
     J.gamma_out = outs[j].gamma;
     J.heat = outs[j].heat;
+    if (failed) return;                           // the run fails and no result is written
     finalize_cells(J, blockIdx.x - J.block0, jobs[j + 1].block0 - J.block0);
 }
 
@@ -337,8 +340,10 @@ int launch_check_fields(const double* nh, const double* x, int64_t ncell, double
     return 1;
 }
 
-int launch_prepare_kappa(const FieldJob& j, bool fp32, cudaStream_t s)
+int launch_prepare_kappa(const FieldJob& job, bool fp32, cudaStream_t s)
 {
+    FieldJob j = job;
+    j.n_th = ordered_threshold(j.n_th);
     if (fp32) prepare_kappa_kernel<float><<<(int)tiles_for(j.ncell), kBlock, 0, s>>>(j);
     else prepare_kappa_kernel<double><<<(int)tiles_for(j.ncell), kBlock, 0, s>>>(j);
     return 1;

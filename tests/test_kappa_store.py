@@ -14,12 +14,12 @@ def dev(tmp_path_factory):
     body = "".join(definition(src, s) for s in ("__device__ __forceinline__ long long bits_of(",
                                                 "__device__ __forceinline__ float narrow(",
                                                 "__device__ __forceinline__ R stored_kappa(",
-                                                "__device__ __forceinline__ long long threshold_bits(",
+                                                "inline double ordered_threshold(",
                                                 "__device__ __forceinline__ bool eligible("))
     return compile_host(tmp_path_factory.mktemp("kappa"), body + """
 extern "C" void f32(const double* k, int n, int elig, float* out) { for (int i = 0; i < n; ++i) out[i] = stored_kappa<float>(k[i], elig); }
 extern "C" void f64(const double* k, int n, int elig, double* out) { for (int i = 0; i < n; ++i) out[i] = stored_kappa<double>(k[i], elig); }
-extern "C" int elig(double nh, double x, double n_th) { return eligible(nh, (1.0 - x) * nh, threshold_bits(n_th)); }
+extern "C" int elig(double nh, double x, double n_th) { return eligible(nh, (1.0 - x) * nh, ordered_threshold(n_th)); }
 """)
 
 
